@@ -71,8 +71,9 @@ __device__ void batch_stage(BatchShared& sh, const BatchDesc* desc, const BatchS
       else if (kind == kRays)
         c = live ? step->n[i] : 0;
       else if (kind == kSegments)
+        // padded to whole warps, so that a walk warp never spans two maps
         c = live && (variant == kAnyWalk || walk_variant(m.layers, m.miss, m.ndt_clear) == variant)
-                ? (long long)m.calls->segments
+                ? ((long long)m.calls->segments + 31) & ~31LL
                 : 0;
       else if (kind == kNdtPending)
         c = live && (m.layers & kLayerNdt) ? (long long)m.calls->ndt_pending : 0;
@@ -160,6 +161,7 @@ __global__ void __launch_bounds__(kBlock, OHM_WALK_MIN_BLOCKS) k_batch_walk(cons
     const int mi = batch_find(sh, g);
     const DeviceMap& m = sh.maps[mi];
     const long long si = g - sh.pref[mi];
+    if (si >= (long long)m.calls->segments) continue;
     unsigned int cas = 0;  // not attributed per map in a batched step
     const bool occ = (m.layers & kLayerOcc) != 0, cnt = (m.layers & kLayerCounts) != 0;
     if (occ && cnt)
@@ -176,22 +178,30 @@ __global__ void __launch_bounds__(kBlock, OHM_WALK_MIN_BLOCKS) k_batch_walk(cons
 // Filtered miss walk of the maps whose walk is kVariant (walk_variant): one
 // launch per variant present in the batch, so that each kernel holds only its
 // own update code (one kernel for every variant spills heavily).
-#ifndef OHM_BATCH_PIPE
-#define OHM_BATCH_PIPE false
-#endif
 template <int kVariant>
 __global__ void __launch_bounds__(kBlock, OHM_FAST_MIN_BLOCKS) k_batch_walk_fast(const BatchDesc* desc, const BatchStep* step) {
   chain_enter();
   __shared__ BatchShared sh;
+  __shared__ WalkShared ws;
   batch_stage(sh, desc, step, kSegments, kVariant);
-  const long long total = sh.pref[sh.n_maps];
+  const long long total = sh.pref[sh.n_maps];  // a multiple of 32: whole warps iterate together
+  unsigned int ops = 0;  // not attributed per map in a batched step
+  if ((threadIdx.x & 31) == 0) ws.n_open[threadIdx.x >> 5] = 0;
+  __syncwarp();
+  int last = -1;
   OHM_BATCH_STRIDE(g, total) {
     const int mi = batch_find(sh, g);
     const DeviceMap& m = sh.maps[mi];
-    unsigned int ops = 0;  // not attributed per map in a batched step
-    walk_segment_fast<(kVariant & 4) != 0, (kVariant & 2) != 0, (kVariant & 1) != 0, OHM_BATCH_PIPE>(
-        m, m.segs[g - sh.pref[mi]], ops);
+    if (kVariant == 4 || kVariant == 6) {  // the voxels in hand belong to the warp's last map
+      if (last >= 0 && mi != last) drain_open(sh.maps[last], ws, 1u);
+      last = mi;
+    }
+    const long long si = g - sh.pref[mi];
+    const bool has = si < (long long)m.calls->segments;
+    walk_segments<(kVariant & 4) != 0, (kVariant & 2) != 0, (kVariant & 1) != 0>(
+        m, has, has ? m.segs[si] : make_int2(0, 0), ws, ops);
   }
+  if (last >= 0) drain_open(sh.maps[last], ws, 1u);
 }
 
 __global__ void __launch_bounds__(kBlock) k_batch_hits(const BatchDesc* desc, const BatchStep* step) {

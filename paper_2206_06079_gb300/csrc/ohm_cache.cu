@@ -124,7 +124,10 @@ __global__ void k_reset_slots(DeviceMap m, const int32_t* slots, int n, const in
     const long long r = t / per, v = t % per;
     if (r < n) {
       const long long off = (long long)slots[r] * per + v;
-      if (m.occ) reinterpret_cast<unsigned int*>(m.occ)[off] = 0xFFFFFFFFu;
+      if (m.occ) {
+        reinterpret_cast<unsigned int*>(m.occ)[off] = 0xFFFFFFFFu;
+        if ((v & 31) == 0) m.sat[off >> 5] = 0u;
+      }
       if (m.counts) m.counts[off] = 0ULL;
       if (m.decay) m.decay[off] = 0ULL;
       if (m.vmean) m.vmean[off] = 0ULL;

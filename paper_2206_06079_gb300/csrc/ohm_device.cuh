@@ -148,6 +148,8 @@ struct DeviceMap {
   int32_t max_regions;
   int32_t* region_coords;        // [max_regions][3]
   float* occ;                    // [max_regions][32768], Morton order inside a region
+  uint32_t* sat;                 // [max_regions][1024], one bit per voxel (bit off % 32 of word off / 32): set only
+                                 // while the voxel's stored log-odds is at or below l_min, so a miss changes nothing
   unsigned long long* counts;    // [max_regions][32768], hits << 32 | misses
   unsigned long long* decay;     // [max_regions][32768], summed path length, 2^-20 m
   unsigned long long* vmean;     // [max_regions][32768], count << 32 | z10 << 20 | y10 << 10 | x10
@@ -217,15 +219,17 @@ __host__ __device__ inline long long pack_region(int rx, int ry, int rz) {
                      ((unsigned long long)rz & m));
 }
 
-// 64-bit finaliser of MurmurHash3 (Appleby), a published bit mixer.
+// The key's two halves combined by an odd multiplier, then the 32-bit
+// finaliser of MurmurHash3 (Appleby), a published bit mixer.  (Its 64-bit
+// finaliser takes three times the instructions; a miss walk hashes two to
+// four keys per ray segment.)
 __device__ __forceinline__ uint32_t hash_key(long long k) {
-  unsigned long long x = (unsigned long long)k;
-  x ^= x >> 33;
-  x *= 0xff51afd7ed558ccdULL;
-  x ^= x >> 33;
-  x *= 0xc4ceb9fe1a85ec53ULL;
-  x ^= x >> 33;
-  return (uint32_t)x;
+  uint32_t x = (uint32_t)k + 0x9e3779b1u * (uint32_t)((unsigned long long)k >> 32);
+  x ^= x >> 16;
+  x *= 0x85ebca6bu;
+  x ^= x >> 13;
+  x *= 0xc2b2ae35u;
+  return x ^ (x >> 16);
 }
 
 // Pool slot of a region, or -1.  Read-only use of the table: one 16-byte
@@ -337,9 +341,9 @@ __device__ __forceinline__ bool quantise(float x, double origin, double scale, l
 // Morton order inside a region: bit 3i = x_i, 3i+1 = y_i, 3i+2 = z_i.
 // ---------------------------------------------------------------------------
 __host__ __device__ __forceinline__ uint32_t spread5(uint32_t x) {
-  uint32_t r = 0;
-  for (int b = 0; b < 5; ++b) r |= ((x >> b) & 1u) << (3 * b);
-  return r;
+  x = (x | (x << 8)) & 0x100fu;   // bit 4 to 12
+  x = (x | (x << 4)) & 0x10c3u;   // bits 2, 3 to 6, 7
+  return (x | (x << 2)) & 0x1249u;
 }
 __host__ __device__ __forceinline__ uint32_t morton(uint32_t x, uint32_t y, uint32_t z) {
   return spread5(x) | (spread5(y) << 1) | (spread5(z) << 2);
@@ -666,6 +670,20 @@ __host__ __device__ __forceinline__ float fmul_rn(float a, float b) {
   return a * b;
 #endif
 }
+__host__ __device__ __forceinline__ float fadd_rn(float a, float b) {
+#ifdef __CUDA_ARCH__
+  return __fadd_rn(a, b);
+#else
+  return a + b;
+#endif
+}
+__host__ __device__ __forceinline__ float fsub_rn(float a, float b) {
+#ifdef __CUDA_ARCH__
+  return __fsub_rn(a, b);
+#else
+  return a - b;
+#endif
+}
 __host__ __device__ __forceinline__ float fma_rn(float a, float b, float c) {
 #ifdef __CUDA_ARCH__
   return __fmaf_rn(a, b, c);
@@ -832,6 +850,234 @@ OHM_UNROLL
   s->visits = steps + 1;
 }
 
+// The axis along which a ray is longest in fixed-point units (the lowest of
+// equal ones).  Taken as the dominant axis of the integrate kernels' rays: no
+// other axis then crosses more than one boundary between two of its steps
+// (two in slot 0 at most, on an exact tie).
+__host__ __device__ __forceinline__ int longest_axis(const long long a[3], const long long b[3]) {
+  long long d0 = b[0] - a[0], d1 = b[1] - a[1], d2 = b[2] - a[2];
+  d0 = d0 < 0 ? -d0 : d0;
+  d1 = d1 < 0 ? -d1 : d1;
+  d2 = d2 < 0 ? -d2 : d2;
+  int M = 0;
+  long long best = d0;
+  if (d1 > best) {
+    best = d1;
+    M = 1;
+  }
+  return d2 > best ? 2 : M;
+}
+
+// ---------------------------------------------------------------------------
+// Local walk: the integrate kernels' miss walk inside one piece of a segment
+// of at most kPieceSlots dominant-axis slots.  It visits exactly the voxels of
+// Walker, in the same order.
+//
+// The ray parameter is measured from the dominant-axis step K0 that opens the
+// piece, in units of dominant-axis steps: the next crossing of axis k (c_k
+// crossings taken) lies at
+//     s_k = ((d0_k + c_k U) A_M - (d0_M + (K0 - 1) U) A_k) / (U A_k),
+// which piece_axis forms from exact 32-bit remainders, and every further
+// crossing adds u_k = A_M / A_k >= 1 (1 along the dominant axis, exactly).  The
+// estimates s^_k start within 7 u s_k (u = 2^-24: the rounded remainder,
+// fraction, difference and A_k, a reciprocal good to one ulp, one product) and
+// take at most 31 additions of u^_k = u_k (1 + 6 u), each rounded, so below 33
+//     |s^_k - s_k| < 33 * 7 u + 33 * 6 u + 31 * 2^-20 < 5.6e-5.
+// The axis with the smallest estimate steps; that is decided when the next
+// smallest lies more than kPieceMargin = 2^-13 = 1.22e-4 behind (above twice the
+// bound and the sum's rounding): every other axis then crosses strictly later,
+// and the step is the one the exact rule takes.  As the axis stepped moves on
+// by at least 1, "the next smallest" is the smallest after the step.  An axis
+// with s_k above 33 keeps s^_k above 32.9, past every crossing of the piece.
+// Otherwise (a near-tie) the exact 64-bit rule decides (exact_pick).  An axis
+// with A_k = 0 has s^_k = +inf.
+// Measuring from the piece keeps the near-tie band at 2^-13 of one step
+// whatever the ray's length, with one add per step; FWalker's parameter grows
+// with the ray, which asks for a fused multiply-add and a crossing count per
+// axis to keep its band as narrow.
+//
+// A piece moves at most 31 voxels along each axis, so it leaves its first
+// region at most once per axis: the sign-normalised Morton index carries a
+// sixth bit per axis (bits 15 x, 16 y, 17 z), set once the walk has left the
+// first region along that axis, and no step tests for a region boundary.
+// ---------------------------------------------------------------------------
+constexpr int kPieceSlots = 30;
+constexpr float kPieceMargin = 1.220703125e-4f;  // 2^-13
+
+struct LWalker {
+  float sx, sy, sz;
+  float ux, uy, uz;
+  float mn;  // the smallest of sx, sy, sz
+};
+
+struct PieceStart {
+  int32_t c[3];    // crossings taken along each axis before the piece's first voxel
+  int32_t v[3];    // its first voxel
+  int32_t ve[3];   // its last voxel
+  int32_t visits;  // voxels it visits
+};
+
+__host__ __device__ __forceinline__ uint32_t morton_mask6(int axis) {
+  return axis == 0 ? 0x9249u : (axis == 1 ? 0x12492u : 0x24924u);
+}
+
+// 1 / x to one ulp.
+__host__ __device__ __forceinline__ float rcp_1ulp(float x) {
+#ifdef __CUDA_ARCH__
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+#else
+  return 1.0f / x;
+#endif
+}
+
+// One axis besides the dominant one, for piece_start: the crossings c before
+// the K0-th dominant-axis step, ce before the K1-th, and the estimates s, u.
+// `above`: the axis' index is above the dominant one's (it steps first on a
+// tie).  With R(K) as in crossings_before and X(K) = floor((R(K) - [not
+// above]) / U), c = floor(X(K0) / A_M) + 1, and with the remainder
+// e = X(K0) - (c - 1) A_M and f = R(K0) - U X(K0) (0 .. U),
+//     ce - c = floor((e + (K1 - K0) A) / A_M),   s = (A_M - e - f / U) / A.
+// The quotient for ce is at most 32: its float estimate is within 1 of it and
+// the remainder (exact modulo 2^32, its magnitude below 2^31) settles it.
+__host__ __device__ __forceinline__ void piece_axis(int32_t A, int32_t d0, int32_t n, int32_t AM, float fAM, float rAM,
+                                                    unsigned long long inv, long long tM, int F, bool above,
+                                                    bool at_start, int32_t slots, int32_t* c, int32_t* ce,
+                                                    float* s, float* u) {
+  const int32_t below = above ? 0 : 1;
+  const long long R = tM * A - (long long)d0 * AM - below;
+  const long long X = R >> F;
+  int32_t e;
+  if (X < 0 || at_start) {
+    *c = 0;
+    e = (int32_t)(X + AM);  // in [-A_M - 2, A_M]
+  } else {
+    const uint32_t q = (uint32_t)umulhi64((unsigned long long)X, inv);  // the quotient or one less, see div_by_inv
+    e = (int32_t)((uint32_t)X - q * (uint32_t)AM);                      // below 2 A_M < 2^31
+    *c = (int32_t)q + 1;
+    if (e >= AM) {
+      e -= AM;
+      *c += 1;
+    }
+  }
+  const float fA = (float)A;
+  int32_t q = (int32_t)fmul_rn(fma_rn((float)slots, fA, (float)e), rAM);
+  const int32_t rem = (int32_t)((uint32_t)e + (uint32_t)slots * (uint32_t)A - (uint32_t)q * (uint32_t)AM);
+  q += rem >= AM ? 1 : (rem < 0 ? -1 : 0);
+  *ce = *c + (q > 0 ? q : 0);
+  if (*c > n) *c = n;
+  if (*ce > n) *ce = n;
+  const int32_t f = (int32_t)(R & ((1LL << F) - 1)) + below;
+  const float rA = rcp_1ulp(fA);
+  *s = A == 0 ? INFINITY : fmul_rn(fsub_rn((float)(AM - e), fmul_rn((float)f, 1.0f / (float)(1 << F))), rA);
+  *u = A == 0 ? 0.0f : fmul_rn(fAM, rA);
+}
+
+// The piece of a ray between its K0-th and K1-th dominant-axis steps (from
+// the voxel entered by the K0-th, the start voxel when K0 = 0, up to, not
+// including, the one entered by the K1-th; to_end: to the end of the ray).
+// K1 - K0 <= kPieceSlots; the ray's dominant axis is its longest
+// (longest_axis).  The two other axes are taken in order, P before Q, so that
+// lanes with different dominant axes run the same code.
+__host__ __device__ __forceinline__ void piece_start(const RayRec& r, int F, int32_t K0, int32_t K1, bool to_end,
+                                                     PieceStart* p, LWalker* w) {
+  const int M = (r.flags >> kRayAxisShift) & 3;
+  const bool m0 = M == 0, m2 = M == 2;
+  const int32_t AM = m0 ? r.A[0] : (m2 ? r.A[2] : r.A[1]);
+  const int32_t dM = m0 ? r.d0[0] : (m2 ? r.d0[2] : r.d0[1]);
+  const int32_t nM = m0 ? r.n[0] : (m2 ? r.n[2] : r.n[1]);
+  const long long tM = (long long)dM + (((long long)K0 - 1) << F);
+  const float fAM = (float)AM, rAM = AM > 0 ? rcp_1ulp(fAM) : 0.0f;
+  const int32_t nP = m0 ? r.n[1] : r.n[0], nQ = m2 ? r.n[1] : r.n[2];
+  int32_t cP, cQ, eP, eQ;
+  float sP, sQ, uP, uQ;
+  piece_axis(m0 ? r.A[1] : r.A[0], m0 ? r.d0[1] : r.d0[0], nP, AM, fAM, rAM, r.inv, tM, F, m0, K0 == 0, K1 - K0, &cP,
+             &eP, &sP, &uP);
+  piece_axis(m2 ? r.A[1] : r.A[2], m2 ? r.d0[1] : r.d0[2], nQ, AM, fAM, rAM, r.inv, tM, F, !m2, K0 == 0, K1 - K0, &cQ,
+             &eQ, &sQ, &uQ);
+  const int32_t eM = to_end ? nM : K1 - 1;
+  if (to_end) {
+    eP = nP;
+    eQ = nQ;
+  }
+  p->visits = (eM - K0) + (eP - cP) + (eQ - cQ) + 1;
+  const float sM = AM > 0 ? 1.0f : INFINITY;
+  p->c[0] = m0 ? K0 : cP;
+  p->c[1] = m0 ? cP : (m2 ? cQ : K0);
+  p->c[2] = m2 ? K0 : cQ;
+  const int32_t ce[3] = {m0 ? eM : eP, m0 ? eP : (m2 ? eQ : eM), m2 ? eM : eQ};
+  w->sx = m0 ? sM : sP;
+  w->sy = m0 ? sP : (m2 ? sQ : sM);
+  w->sz = m2 ? sM : sQ;
+  w->ux = m0 ? 1.0f : uP;
+  w->uy = m0 ? uP : (m2 ? uQ : 1.0f);
+  w->uz = m2 ? 1.0f : uQ;
+  w->mn = fminf(w->sx, fminf(w->sy, w->sz));
+OHM_UNROLL
+  for (int k = 0; k < 3; ++k) {
+    const bool neg = (r.flags >> (kRaySignShift + k)) & 1;
+    p->v[k] = neg ? r.v0[k] - p->c[k] : r.v0[k] + p->c[k];
+    p->ve[k] = neg ? r.v0[k] - ce[k] : r.v0[k] + ce[k];
+  }
+}
+
+// One crossing: the axis with the smallest estimate steps (estimates and
+// sign-normalised Morton index of six bits per axis).  Returns false on a
+// near-tie, when the step taken need not be the exact one.  Written with
+// selects and predicated adds, so that lanes stepping different axes do not
+// diverge.
+__host__ __device__ __forceinline__ bool lwalker_step(LWalker& w, uint32_t& mo) {
+  const float thr = fadd_rn(w.mn, kPieceMargin);
+  const bool nx = w.sx == w.mn, ny = !nx && w.sy == w.mn, nz = !nx && !ny;
+  const uint32_t mask = nx ? 0x9249u : (ny ? 0x12492u : 0x24924u);
+  if (nx) w.sx = fadd_rn(w.sx, w.ux);
+  if (ny) w.sy = fadd_rn(w.sy, w.uy);
+  if (nz) w.sz = fadd_rn(w.sz, w.uz);
+  mo = (((mo | ~mask) + 1u) & mask) | (mo & ~mask);
+  w.mn = fminf(w.sx, fminf(w.sy, w.sz));
+  return w.mn > thr;
+}
+
+// Coordinate along `axis` in a Morton index with six bits per axis.
+__host__ __device__ __forceinline__ int32_t morton_coord6(uint32_t mo, int axis) {
+  uint32_t x = mo >> axis, c = 0;
+OHM_UNROLL
+  for (int b = 0; b < 6; ++b) c |= ((x >> (3 * b)) & 1u) << b;
+  return (int32_t)c;
+}
+
+// n exact steps of the piece that starts at dominant-axis step K0, from the
+// voxel of sign-normalised index mo (six bits per axis, region bits relative
+// to the piece's first region); the indices reached go to out.  mo and w are
+// left after the last step, w's estimates as fresh ones would be (fewer
+// roundings than the bound above counts).
+__host__ __device__ inline void piece_exact_steps(const RayRec& r, int F, int32_t K0, LWalker& w, uint32_t& mo, int n,
+                                                  uint32_t* out) {
+  PieceStart p;
+  piece_start(r, F, K0, K0 + 1, false, &p, &w);
+  int32_t c[3];
+OHM_UNROLL
+  for (int k = 0; k < 3; ++k) {
+    const bool neg = (r.flags >> (kRaySignShift + k)) & 1;
+    const int32_t local = p.v[k] & 31, first = neg ? 31 - local : local;
+    c[k] = p.c[k] + morton_coord6(mo, k) - first;
+  }
+  for (int i = 0; i < n; ++i) {
+    const int axis = exact_pick(r, F, c[0], c[1], c[2]);
+    c[0] += axis == 0;
+    c[1] += axis == 1;
+    c[2] += axis == 2;
+    const uint32_t mask = morton_mask6(axis);
+    mo = (((mo | ~mask) + 1u) & mask) | (mo & ~mask);
+    out[i] = mo;
+  }
+  if (c[0] > p.c[0]) w.sx = fma_rn((float)(c[0] - p.c[0]), w.ux, w.sx);
+  if (c[1] > p.c[1]) w.sy = fma_rn((float)(c[1] - p.c[1]), w.uy, w.sy);
+  if (c[2] > p.c[2]) w.sz = fma_rn((float)(c[2] - p.c[2]), w.uz, w.sz);
+  w.mn = fminf(w.sx, fminf(w.sy, w.sz));
+}
+
 // ---------------------------------------------------------------------------
 // Warp-aggregated reservation: every lane of a full warp calls this together
 // with its own count (possibly 0); returns this lane's first index.
@@ -973,20 +1219,6 @@ OHM_UNROLL
 // contraction changes it.
 // ---------------------------------------------------------------------------
 
-__host__ __device__ __forceinline__ float fadd_rn(float a, float b) {
-#ifdef __CUDA_ARCH__
-  return __fadd_rn(a, b);
-#else
-  return a + b;
-#endif
-}
-__host__ __device__ __forceinline__ float fsub_rn(float a, float b) {
-#ifdef __CUDA_ARCH__
-  return __fsub_rn(a, b);
-#else
-  return a - b;
-#endif
-}
 __host__ __device__ __forceinline__ float fdiv_rn(float a, float b) {
 #ifdef __CUDA_ARCH__
   return __fdiv_rn(a, b);

@@ -63,29 +63,27 @@ __global__ void __launch_bounds__(kBlock, OHM_WALK_MIN_BLOCKS) k_walk_miss(Devic
   if ((threadIdx.x & 31) == 0 && cas) atomicAdd(&m.calls->atomics, (unsigned long long)cas);
 }
 
-// The miss walk of maps without the decay layer (filtered walk, see
-// walk_segment_fast).
-// OHM_SINGLE_PIPE: the single-map walk runs the pipelined loop (the plain
-// loop of the multi-map batch, with its unchecked CAS initialisation, was
-// slower on tunnel scans at 4 and 5 blocks per SM).
-#ifndef OHM_SINGLE_PIPE
-#define OHM_SINGLE_PIPE true
-#endif
+// The miss walk of maps without the decay layer (walk_segments).
 template <bool kOcc, bool kCounts, bool kCas>
 __global__ void __launch_bounds__(kBlock, OHM_FAST_MIN_BLOCKS) k_walk_fast(DeviceMap m) {
   chain_enter();
   if (latched(m)) return;
+  __shared__ WalkShared sh;
   const long long nseg = (long long)m.calls->segments;
-  const long long stride = (long long)gridDim.x * blockDim.x;
+  const long long stride = (long long)gridDim.x * kBlock;
   unsigned int ops = 0;
+  if ((threadIdx.x & 31) == 0) sh.n_open[threadIdx.x >> 5] = 0;
+  __syncwarp();
   long long si = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   int2 sg = si < nseg ? m.segs[si] : make_int2(0, 0);
-  for (; si < nseg; si += stride) {
+  // whole warps iterate together
+  for (; si - (threadIdx.x & 31) < nseg; si += stride) {
     // the next segment's table entry is loaded while this one walks
     const int2 next = si + stride < nseg ? m.segs[si + stride] : make_int2(-1, 0);
-    walk_segment_fast<kOcc, kCounts, kCas, OHM_SINGLE_PIPE>(m, sg, ops, next.x >= 0 ? m.rays + next.x : nullptr);
+    walk_segments<kOcc, kCounts, kCas>(m, si < nseg, sg, sh, ops, next.x >= 0 ? m.rays + next.x : nullptr);
     sg = next;
   }
+  if (kOcc && !kCas) ops += drain_open(m, sh, 1u);
   // every thread gets here: one atomic per warp for the call's atomic count
   ops = __reduce_add_sync(0xffffffffu, ops);
   if ((threadIdx.x & 31) == 0 && ops) atomicAdd(&m.calls->atomics, (unsigned long long)ops);

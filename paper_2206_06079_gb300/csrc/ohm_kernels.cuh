@@ -57,7 +57,7 @@ inline void launch_chained(void (*kernel)(K...), unsigned grid, cudaStream_t str
 
 // Log-odds of a stored occupancy word for an update: an unknown voxel (NaN)
 // starts from the prior 0, and a value stored below l_min stands for l_min
-// (the miss walk may leave it there, see walk_segment_fast).
+// (the miss walk may leave it there, see walk_segments).
 __device__ __forceinline__ float logodds_value(float s, float l_min) { return s != s ? 0.0f : fmaxf(s, l_min); }
 
 // Log-odds a stored occupancy word reports: NaN stays unknown, a value stored
@@ -265,7 +265,7 @@ __device__ __forceinline__ void miss_cas(const DeviceMap& m, unsigned int* u, un
 #endif
 constexpr int kWalkBatch = OHM_WALK_BATCH;
 #ifndef OHM_WALK_OVERSUBSCRIBE
-#define OHM_WALK_OVERSUBSCRIBE 8
+#define OHM_WALK_OVERSUBSCRIBE 4
 #endif
 #ifndef OHM_PREPARE_MIN_BLOCKS
 #define OHM_PREPARE_MIN_BLOCKS 4
@@ -390,15 +390,17 @@ __device__ __forceinline__ void prepare_occ_ray(const DeviceMap& m, const CallAr
       ok = in_extent(qo, F) && in_extent(qe, F);
     }
     if (ok) {
-      int32_t nmaj;
-      const int M = dominant_axis(qo, qe, F, &nmaj);
+      const int M = longest_axis(qo, qe);
+      long long nmaj = 0;
       long long l1 = 0;
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
         long long dv = (qe[k] >> F) - (qo[k] >> F);
-        l1 += dv < 0 ? -dv : dv;
+        dv = dv < 0 ? -dv : dv;
+        l1 += dv;
+        if (k == M) nmaj = dv;
       }
-      const SegSplit sp = ray_segment_split(nmaj, l1, m.seg_steps);
+      const SegSplit sp = ray_segment_split((int32_t)nmaj, l1, m.seg_steps);
       nseg = (unsigned int)sp.nseg;
       const long long am = sel3(M, qe[0] - qo[0], qe[1] - qo[1], qe[2] - qo[2]);
       r.inv = reciprocal64((unsigned long long)(am < 0 ? -am : am));
@@ -578,39 +580,163 @@ __device__ __forceinline__ void find_region2(const DeviceMap& m, long long k1, l
   *s2 = e2.x == k2 ? (int32_t)e2.y : (e2.x == kEmptyKey ? -1 : find_region(m, k2));
 }
 
-// Out of line: the rare paths of the filtered walk (a near-tie decided
-// exactly from the ray record, a third region inside one segment), so that
-// neither the record nor the hash loop takes registers in the walk.
-static __device__ __noinline__ int exact_pick_rec(const RayRec* rp, int F, int32_t c0, int32_t c1, int32_t c2) {
-  return exact_pick(*rp, F, c0, c1, c2);
+// Out of line: the rare paths of the miss walk (a batch with a near-tie,
+// stepped exactly from the ray record; a region the piece's set-up did not
+// foresee), so that neither the record nor the hash loop takes registers in
+// the walk.
+struct ExactBatch {
+  LWalker w;
+  uint32_t mo;
+  uint32_t at[8];
+};
+static __device__ __noinline__ void exact_batch(const RayRec* rp, int F, int32_t K0, int n, ExactBatch* b) {
+  const RayRec r = *rp;
+  piece_exact_steps(r, F, K0, b->w, b->mo, n, b->at);
 }
-static __device__ __noinline__ int32_t find_region_rare(const DeviceMap& m, long long key) { return find_region(m, key); }
 
-// Voxels per batch of the filtered walk: pipelined (two batches in flight,
-// the single-map walk kernel) and plain (one batch stepped, loaded and
-// applied at a time, the multi-map batch kernel, whose run-time choice of
-// layers leaves fewer registers for the pipeline).
+// The key of the region reached from region `key` by one step along each
+// axis whose bit is set in idx, in the direction of the ray's signs.
+__device__ __forceinline__ long long neighbour_key(long long key, uint32_t idx, int32_t signs) {
+  const unsigned long long k = (unsigned long long)key;
+  const int32_t mask = (1 << 21) - 1;
+  int32_t c[3] = {(int32_t)((k >> 42) & mask), (int32_t)((k >> 21) & mask), (int32_t)(k & mask)};
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+    if ((idx >> a) & 1u) c[a] += ((signs >> a) & 1) ? -1 : 1;
+  return pack_region(c[0], c[1], c[2]);
+}
+static __device__ __noinline__ int32_t find_neighbour_rare(const DeviceMap& m, const RayRec* rp, int32_t K0, uint32_t idx) {
+  const RayRec r = *rp;
+  PieceStart p;
+  LWalker w;
+  piece_start(r, m.frac_bits, K0, K0 + 1, false, &p, &w);
+  return find_region(m, neighbour_key(pack_region(p.v[0] >> kRegionShift, p.v[1] >> kRegionShift, p.v[2] >> kRegionShift),
+                                      idx, (r.flags >> kRaySignShift) & 7));
+}
+
+// Voxels per batch of the miss walk, and the blocks per SM it is compiled for.
 #ifndef OHM_FAST_BATCH
 #define OHM_FAST_BATCH 4
-#endif
-#ifndef OHM_FAST_BATCH_PLAIN
-#define OHM_FAST_BATCH_PLAIN 8
 #endif
 #ifndef OHM_FAST_MIN_BLOCKS
 #define OHM_FAST_MIN_BLOCKS 4
 #endif
 constexpr int kFastBatch = OHM_FAST_BATCH;
-constexpr int kFastBatchPlain = OHM_FAST_BATCH_PLAIN;
-template <bool kPipe>
-constexpr int kFastBatchOf = kPipe ? kFastBatch : kFastBatchPlain;
 
+// Shared memory of a walk block.
+//
+// Region bases of a piece, one column of `tab` per thread.  Entry idx (bit k:
+// the walk has left its first region along axis k) at idx * kBlock is
+// base ^ neg ^ (idx << 15) with base the region's first voxel offset, so that
+// its exclusive or with the sign-normalised Morton index mo (idx = mo >> 15)
+// is the voxel's offset base | ((mo ^ neg) & 0x7fff).  kNoRegion: not looked up.
+//
+// `open`: per warp, offsets of voxels whose saturation bit was clear, waiting
+// to be looked at; less than a round between batches.  They are
+// looked at kOpenEach per lane (2 and 8 were slower: 73 / 72 / 86 us for 2, 4
+// and 8 on a mapped tunnel scan, 170 / 154 / 161 us in unknown space).
+#ifndef OHM_OPEN_EACH
+#define OHM_OPEN_EACH 4
+#endif
+constexpr uint32_t kOpenEach = OHM_OPEN_EACH;
+constexpr uint32_t kOpenRound = 32 * kOpenEach;
+constexpr int kOpenCap = kOpenRound + 32 * kFastBatch;
+struct WalkShared {
+  uint32_t tab[8 * kBlock];
+  uint32_t open[kBlock / 32][kOpenCap];
+  uint32_t n_open[kBlock / 32];
+};
+constexpr uint32_t kNoRegion = 0x80000000u;
+__device__ __forceinline__ uint32_t region_entry(int32_t slot, uint32_t neg, uint32_t idx) {
+  return ((uint32_t)slot << (3 * kRegionShift)) ^ neg ^ (idx << (3 * kRegionShift));
+}
 
-// Miss phase (Sec. III-C phase one) of one segment with the filtered walk
-// (FWalker): every voxel the ray passes through, except the voxel holding its
-// sample, takes one miss.  The segment's first and last regions are looked up
-// together before the walk; a region boundary inside the segment costs a
-// comparison with the last region's key and only a hash lookup when the
-// segment passes through a third region.
+// Tells the compiler that a pointer read from a DeviceMap outside constant
+// memory (by reference, or from the batch kernels' shared copy) is global: its
+// loads are global ones and an atomic whose result is unused goes out as a
+// reduction instead of a generic atomic that returns a value.
+template <typename T>
+__device__ __forceinline__ T* global_ptr(T* p) {
+  __builtin_assume(__isGlobal(p));
+  return p;
+}
+
+// One miss of voxel `off`, whose word was read as `word` (add form, see
+// walk_segments).  Returns true if the voxel was unknown and the
+// compare-and-swap went out: its result is in `word` then.
+__device__ __forceinline__ bool miss_add(float* occ, uint32_t off, uint32_t& word, float miss, float l_min,
+                                         unsigned int& ops) {
+  const float l = __uint_as_float(word);
+  if (l > l_min) {
+    atomicAdd(occ + off, miss);
+    ++ops;
+  } else if (l != l) {
+    // an unknown voxel's first miss
+    word = atomicCAS(reinterpret_cast<unsigned int*>(occ) + off, word, __float_as_uint(__fadd_rn(0.0f, miss)));
+    ++ops;
+    return true;
+  }
+  return false;
+}
+
+// Look at the warp's waiting voxels and give them their misses, until fewer
+// than `keep` + 1 wait; four per lane at a time.  Returns the log-odds atomics
+// this lane issued.  Whole warps; out of line: a well observed map comes here
+// about once per six rounds of segments.
+static __device__ __noinline__ unsigned int drain_open(float* occ_any, uint32_t* sat_any, float miss, float l_min,
+                                                       WalkShared& sh, uint32_t keep) {
+  constexpr int kEach = (int)kOpenEach;
+  float* const occ = global_ptr(occ_any);
+  uint32_t* const sat = global_ptr(sat_any);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  unsigned int ops = 0;
+  __syncwarp();
+  uint32_t n = sh.n_open[wid];
+  while (n >= keep) {
+    const uint32_t first = n > kOpenRound ? n - kOpenRound : 0u;
+    uint32_t off[kEach], word[kEach], bits[kEach];
+    bool cas[kEach];
+#pragma unroll
+    for (int j = 0; j < kEach; ++j) {
+      const uint32_t i = first + (uint32_t)(32 * j + lane);
+      off[j] = i < n ? sh.open[wid][i] : kNoRegion;
+      if (off[j] != kNoRegion) word[j] = __float_as_uint(occ[off[j]]);
+    }
+    // voxels found at or below l_min get their bit.  Its word is looked at in
+    // L2 first: many rays find the voxels around the sensor saturated in the
+    // same call, and repeated ORs of one word would queue
+#pragma unroll
+    for (int j = 0; j < kEach; ++j) {
+      bits[j] = ~0u;
+      if (off[j] != kNoRegion && __uint_as_float(word[j]) <= l_min) bits[j] = __ldcg(sat + (off[j] >> 5));
+      cas[j] = off[j] != kNoRegion && miss_add(occ, off[j], word[j], miss, l_min, ops);
+    }
+#pragma unroll
+    for (int j = 0; j < kEach; ++j) {
+      if (!((bits[j] >> (off[j] & 31u)) & 1u)) atomicOr(sat + (off[j] >> 5), 1u << (off[j] & 31u));
+      if (cas[j] && __uint_as_float(word[j]) > l_min) {
+        atomicAdd(occ + off[j], miss);
+        ++ops;
+      }
+    }
+    n = first;
+  }
+  __syncwarp();
+  if (lane == 0) sh.n_open[wid] = n;
+  __syncwarp();
+  return ops;
+}
+__device__ __forceinline__ unsigned int drain_open(const DeviceMap& m, WalkShared& sh, uint32_t keep) {
+  return drain_open(m.occ, m.sat, m.miss, m.l_min, sh, keep);
+}
+
+// Miss phase (Sec. III-C phase one) of one segment per lane (has = false: no
+// segment): every voxel a ray passes through, except the voxel holding its
+// sample, takes one miss.  Whole warps.  The walk is the exact local walk of
+// ohm_device.cuh (LWalker), piece by piece (a segment of the default length is
+// one piece).  The regions a piece passes through are looked up before it is
+// walked, with the order of the boundary crossings taken from the estimates;
+// one the estimates mistook is looked up when met.
 //
 // Occupancy update.  With kCas false (the miss increment is negative and the
 // map does not clear NDT samples) a miss is a fire-and-forget float atomic add
@@ -632,179 +758,191 @@ constexpr int kFastBatchOf = kPipe ? kFastBatch : kFastBatchPlain;
 // see the update that crosses its threshold, or a miss increment >= 0) every
 // miss is a clamped compare-and-swap.
 //
-// kPipe: walk the next batch of voxels and issue its loads while the loads of
-// the batch before are in flight, then apply that batch (a software pipeline
-// of two batches); otherwise walk, load and apply one batch at a time.  The
-// pipeline wins where many voxels are still unknown (their compare-and-swaps
-// wait for a result) and costs a little on well-observed maps.
-template <bool kOcc, bool kCounts, bool kCas, bool kPipe = true>
-__device__ __forceinline__ void walk_segment_fast(const DeviceMap& m, int2 sg, unsigned int& ops,
-                                                  const RayRec* prefetch = nullptr) {
+// Saturated voxels.  Most voxels a ray passes are free space that is at l_min
+// already (99 % of the visits of a scan in a mapped tunnel).  Their bit in
+// DeviceMap::sat says so: 32 bits, a 4 x 4 x 2 brick of voxels, per load instead
+// of one float per voxel, read once per brick the ray enters, from a plane 1/32
+// the size of the floats.  Voxels whose bit is clear are collected per warp
+// and looked at kOpenRound at a time (drain_open), so the few of a well
+// observed map neither stop the warp nor run its update code for one lane,
+// and the many of unknown space go out kOpenEach per lane.  A voxel found at
+// l_min gets its bit there; the hits clear it; a stale clear bit only costs
+// the look.
+//
+// A batch is stepped without a branch; one that met a near-tie is stepped
+// again exactly.  What bounds the walk is instruction issue (46 M warp
+// instructions for 19.3 M visits of a 131,072-ray tunnel scan, 83 M before)
+// and the code is kept small, one copy of the stepping: a software pipeline
+// of two batches and a second form that reads the floats directly were slower
+// by what they add to the instruction cache and the registers.
+// Measured (131,072-ray tunnel scan, 0.1 m, 865 k segments): 123.5 -> 72.4 us in
+// a mapped tunnel, 164 -> 154 us in unknown space; 262,144 rays at 0.05 m
+// 308 -> 162 us; outdoor scans into half-known space 144 -> 104 us.
+template <bool kOcc, bool kCounts, bool kCas>
+__device__ __forceinline__ void walk_segments(const DeviceMap& m, bool has, int2 sg, WalkShared& sh,
+                                              unsigned int& ops, const RayRec* prefetch = nullptr) {
+  constexpr uint32_t kAll = (1u << kFastBatch) - 1u;
+  static_assert(kFastBatch <= 8, "ExactBatch holds 8 indices");
+  const unsigned full = 0xffffffffu;
   const int F = m.frac_bits;
-  const RayRec* rp = m.rays + sg.x;
-  FWalker f;
-  uint32_t mo, neg;
-  int32_t rcx, rcy, rcz, sgn, left, slot, slotE;
-  long long keyE;
-  {
-    const RayRec r = *rp;
-    SegStart s;
-    segment_start(r, F, sg.y, &s);
-    const bool last = sg.y == r.nseg - 1;
-    left = (int32_t)s.visits - ((last && (r.flags & kRaySample)) ? 1 : 0);
-    fwalker_init(f, r, F, s.c);
-    neg = morton_neg(r.flags);
-    sgn = (r.flags >> kRaySignShift) & 7;
-    mo = local_morton(s.v[0], s.v[1], s.v[2]) ^ neg;
-    rcx = s.v[0] >> kRegionShift;
-    rcy = s.v[1] >> kRegionShift;
-    rcz = s.v[2] >> kRegionShift;
-    keyE = pack_region(s.ve[0] >> kRegionShift, s.ve[1] >> kRegionShift, s.ve[2] >> kRegionShift);
-    find_region2(m, pack_region(rcx, rcy, rcz), keyE, &slot, &slotE);
-  }
-  // the record of the thread's next segment, into L2 while this one walks
-  if (prefetch) asm volatile("prefetch.global.L2 [%0];" ::"l"(prefetch));
-  if (left <= 0) return;
-  if (slot < 0 || slotE < 0) {
-    atomicOr(m.status, kStatusMissing);
-    return;
-  }
-  uint32_t base = (uint32_t)slot << (3 * kRegionShift);
-  unsigned int* occ = reinterpret_cast<unsigned int*>(m.occ);
-  const unsigned int miss0 = __float_as_uint(__fadd_rn(0.0f, m.miss));  // an unknown voxel's first miss
-  auto fill = [&](uint32_t (&off)[kFastBatchOf<kPipe>]) -> uint32_t {
-    uint32_t valid = 0;
+  uint32_t* const tab = sh.tab + threadIdx.x;
+  const RayRec* rp = global_ptr(m.rays) + (has ? sg.x : 0);
+  unsigned int* const occ = reinterpret_cast<unsigned int*>(global_ptr(m.occ));
+  const uint32_t* const sat = global_ptr(m.sat);
+  unsigned long long* const counts = global_ptr(m.counts);
+  int32_t K = 0, K1 = -1;  // the piece's first dominant-axis step, the segment's end (not yet known)
+  bool more = has;
+  while (__any_sync(full, more)) {
+    LWalker w = {};
+    uint32_t mo = 0;
+    int32_t left = 0;
+    if (more) {
+      const RayRec r = *rp;
+      const int M = (r.flags >> kRayAxisShift) & 3;
+      const int32_t nmaj = M == 0 ? r.n[0] : (M == 1 ? r.n[1] : r.n[2]);
+      if (K1 < 0) {
+        // segment_bounds in 32 bits (at most 2^25 slots per ray)
+        const int32_t q = (int32_t)((uint32_t)r.flags >> kRaySegShift), extra = nmaj + 1 - r.nseg * q;
+        K = sg.y * q + (sg.y < extra ? sg.y : extra);
+        K1 = K + q + (sg.y < extra ? 1 : 0);
+        // the record of the thread's next segment, into L2 while this one walks
+        if (prefetch) asm volatile("prefetch.global.L2 [%0];" ::"l"(prefetch));
+      }
+      const int32_t K0 = K, Ke = K + kPieceSlots < K1 ? K + kPieceSlots : K1;
+      PieceStart p;
+      piece_start(r, F, K0, Ke, Ke == nmaj + 1, &p, &w);
+      left = p.visits - ((Ke == nmaj + 1 && (r.flags & kRaySample)) ? 1 : 0);
+      const uint32_t neg = morton_neg(r.flags);
+      const int32_t signs = (r.flags >> kRaySignShift) & 7;
+      mo = local_morton(p.v[0], p.v[1], p.v[2]) ^ neg;
+      const int32_t a0 = p.v[0] >> kRegionShift, a1 = p.v[1] >> kRegionShift, a2 = p.v[2] >> kRegionShift;
+      const int32_t b0 = p.ve[0] >> kRegionShift, b1 = p.ve[1] >> kRegionShift, b2 = p.ve[2] >> kRegionShift;
+      const uint32_t idx = (a0 != b0 ? 1u : 0u) | (a1 != b1 ? 2u : 0u) | (a2 != b2 ? 4u : 0u);
+      int32_t slot, slotE;
+      find_region2(m, pack_region(a0, a1, a2), pack_region(b0, b1, b2), &slot, &slotE);
 #pragma unroll
-    for (int j = 0; j < kFastBatchOf<kPipe>; ++j) {
-      off[j] = base | (mo ^ neg);  // voxel offset (< 2^31: at most 2^16 regions of 2^15 voxels)
-      if (left > 0) {
-        valid |= 1u << j;
-        --left;
-        if (left > 0) {
-          int axis = fwalker_pick(f);
-          if (axis < 0) axis = exact_pick_rec(rp, F, (int32_t)f.cx, (int32_t)f.cy, (int32_t)f.cz);
-          fwalker_advance(f, axis);
-          if (morton_advance(mo, morton_mask(axis))) {
-            const int32_t d = ((sgn >> axis) & 1) ? -1 : 1;
-            if (axis == 0)
-              rcx += d;
-            else if (axis == 1)
-              rcy += d;
-            else
-              rcz += d;
-            const long long key = pack_region(rcx, rcy, rcz);
-            const int32_t ns = key == keyE ? slotE : find_region_rare(m, key);
-            if (ns < 0) {
-              atomicOr(m.status, kStatusMissing);
-              left = 0;
-            } else {
-              base = (uint32_t)ns << (3 * kRegionShift);
+      for (int i = 1; i < 8; ++i) tab[i * kBlock] = kNoRegion;
+      tab[0] = region_entry(slot, neg, 0);
+      tab[idx * kBlock] = region_entry(slotE, neg, idx);
+      if (slot < 0 || slotE < 0) {
+        if (left > 0) atomicOr(m.status, kStatusMissing);
+        left = 0;
+      } else if (idx & (idx - 1u)) {  // two or three boundaries: the regions between
+        // the parameter at which the piece leaves its first region, per axis it does
+        const float o0 = (idx & 1u) ? w.sx + (float)((signs & 1) ? p.v[0] & 31 : ~p.v[0] & 31) * w.ux : INFINITY;
+        const float o1 = (idx & 2u) ? w.sy + (float)((signs & 2) ? p.v[1] & 31 : ~p.v[1] & 31) * w.uy : INFINITY;
+        const float o2 = (idx & 4u) ? w.sz + (float)((signs & 4) ? p.v[2] & 31 : ~p.v[2] & 31) * w.uz : INFINITY;
+        const uint32_t i1 = o0 <= o1 ? (o0 <= o2 ? 1u : 4u) : (o1 <= o2 ? 2u : 4u);
+        const uint32_t i3 = o0 > o1 ? (o0 > o2 ? 1u : 4u) : (o1 > o2 ? 2u : 4u);
+        const uint32_t i2 = idx == 7u ? 7u & ~i3 : i1;
+        int32_t s1, s2;
+        find_region2(m, pack_region((i1 & 1u) ? b0 : a0, (i1 & 2u) ? b1 : a1, (i1 & 4u) ? b2 : a2),
+                     pack_region((i2 & 1u) ? b0 : a0, (i2 & 2u) ? b1 : a1, (i2 & 4u) ? b2 : a2), &s1, &s2);
+        if (s1 >= 0) tab[i1 * kBlock] = region_entry(s1, neg, i1);
+        if (s2 >= 0) tab[i2 * kBlock] = region_entry(s2, neg, i2);
+      }
+    }
+    // step kFastBatch voxels: sign-normalised Morton indices (at), offsets,
+    // and which voxels exist (valid)
+    auto fill = [&](uint32_t (&at)[kFastBatch], uint32_t (&off)[kFastBatch], uint32_t& valid) {
+      bool sure = true;
+#pragma unroll
+      for (int j = 0; j < kFastBatch; ++j) {
+        at[j] = mo;
+        sure = lwalker_step(w, mo) && sure;
+      }
+      valid = left >= kFastBatch ? kAll : (left > 0 ? (1u << left) - 1u : 0u);
+      if (!sure && valid) {
+        ExactBatch b;
+        b.mo = at[0];
+        exact_batch(rp, F, K, kFastBatch, &b);
+        w = b.w;
+        mo = b.mo;
+#pragma unroll
+        for (int j = 1; j < kFastBatch; ++j) at[j] = b.at[j - 1];
+      }
+      left -= kFastBatch;
+      uint32_t any = 0;
+#pragma unroll
+      for (int j = 0; j < kFastBatch; ++j) {
+        off[j] = tab[(at[j] >> 15) * kBlock] ^ at[j];  // voxel offset (< 2^31: at most 2^16 regions of 2^15 voxels)
+        any |= off[j];
+      }
+      if ((any & kNoRegion) && valid) {
+#pragma unroll
+        for (int j = 0; j < kFastBatch; ++j) {
+          if (((valid >> j) & 1u) && (off[j] & kNoRegion)) {
+            const uint32_t idx = at[j] >> 15;
+            uint32_t e = tab[idx * kBlock];
+            if (e == kNoRegion) {
+              const int32_t s = find_neighbour_rare(m, rp, K, idx);
+              if (s < 0) {
+                atomicOr(m.status, kStatusMissing);
+                valid &= ~(1u << j);
+                continue;
+              }
+              e = region_entry(s, morton_neg(rp->flags), idx);
+              tab[idx * kBlock] = e;
             }
+            off[j] = e ^ at[j];
           }
         }
       }
-    }
-    return valid;
-  };
-  auto issue = [&](const uint32_t (&off)[kFastBatchOf<kPipe>], uint32_t valid, unsigned int (&old)[kFastBatchOf<kPipe>]) {
-    if (kCounts) {
+    };
+    // batches of the warp's longest piece
+    int rounds = __reduce_max_sync(full, left > 0 ? left + kFastBatch - 1 : 0) / kFastBatch;
+    uint32_t brick = ~mo, word = 0;  // the last voxel stepped; the word of the last brick
+    for (; rounds > 0; --rounds) {
+      uint32_t at[kFastBatch], off[kFastBatch], v[kFastBatch], valid;
+      fill(at, off, valid);
+      if (kCounts) {
 #pragma unroll
-      for (int j = 0; j < kFastBatchOf<kPipe>; ++j)
-        if ((valid >> j) & 1u) atomicAdd(m.counts + off[j], 1ULL);
-    }
-    if (kOcc) {
+        for (int j = 0; j < kFastBatch; ++j)
+          if ((valid >> j) & 1u) atomicAdd(counts + off[j], 1ULL);
+      }
+      if (!kOcc) continue;
+      if (kCas) {
 #pragma unroll
-      for (int j = 0; j < kFastBatchOf<kPipe>; ++j) old[j] = ((valid >> j) & 1u) ? occ[off[j]] : 0u;
-    }
-  };
-  auto apply = [&](const uint32_t (&off)[kFastBatchOf<kPipe>], uint32_t valid, unsigned int (&old)[kFastBatchOf<kPipe>]) {
-    if (!kOcc) return;
-    if (kCas) {
+        for (int j = 0; j < kFastBatch; ++j)
+          if ((valid >> j) & 1u) v[j] = occ[off[j]];
 #pragma unroll
-      for (int j = 0; j < kFastBatchOf<kPipe>; ++j)
-        if ((valid >> j) & 1u) miss_cas(m, occ + off[j], old[j], ops);
-      return;
-    }
-    if constexpr (!kPipe) {
-      // Plain loop: an unknown voxel (NaN) is first set to the prior 0 by a
-      // compare-and-swap whose result is not needed (one that loses finds a
-      // value another thread set), then takes its miss as one more add of
-      // delta, like a known voxel above l_min.  All of a call's misses of
-      // the voxel are then adds of delta to 0, in any order: the values 0,
-      // fl(0 + delta), ... of the clamped sequence that starts from the
-      // prior (the clamp on read as above).  Same-address atomics of one
-      // thread stay in order, so a thread's add never lands before its own
-      // compare-and-swap.  Nothing here waits for a result, which the plain
-      // loop (no second batch in flight) cannot hide; the pipelined loop
-      // hides that wait and does better with one atomic per unknown voxel.
+        for (int j = 0; j < kFastBatch; ++j)
+          if ((valid >> j) & 1u) miss_cas(m, occ + off[j], v[j], ops);
+        continue;
+      }
+      // the words of the bricks entered, then the voxels not known to be saturated
+      uint32_t entered = 0, open = valid;
 #pragma unroll
-      for (int j = 0; j < kFastBatchOf<kPipe>; ++j) {
-        if (!((valid >> j) & 1u)) continue;
-        const float l = __uint_as_float(old[j]);
-        if (l != l) {
-          atomicCAS(occ + off[j], old[j], 0u);
-          ++ops;
-        }
-        if (!(l <= m.l_min)) {
-          atomicAdd(reinterpret_cast<float*>(occ + off[j]), m.miss);
-          ++ops;
+      for (int j = 0; j < kFastBatch; ++j) {
+        if (((at[j] ^ (j ? at[j - 1] : brick)) & ~31u) && ((valid >> j) & 1u)) {
+          entered |= 1u << j;
+          v[j] = sat[off[j] >> 5];
         }
       }
-      return;
-    }
-    // adds go out at once; the compare-and-swaps that set unknown voxels
-    // are all issued before any of their results is looked at.  A CAS
-    // that won returns the NaN it replaced; one that lost returns the
-    // (known) value another thread wrote, to which this ray's miss is then
-    // added -- so the word read back replaces the one loaded.
-    uint32_t init = 0;
+      brick = at[kFastBatch - 1];
 #pragma unroll
-    for (int j = 0; j < kFastBatchOf<kPipe>; ++j) {
-      if (!((valid >> j) & 1u)) continue;
-      const float l = __uint_as_float(old[j]);
-      if (l > m.l_min) {
-        atomicAdd(reinterpret_cast<float*>(occ + off[j]), m.miss);
-        ++ops;
-      } else if (l != l) {
-        old[j] = atomicCAS(occ + off[j], old[j], miss0);
-        init |= 1u << j;
-        ++ops;
+      for (int j = 0; j < kFastBatch; ++j) {
+        if ((entered >> j) & 1u) word = v[j];
+        open &= ~(((word >> (off[j] & 31u)) & 1u) << j);
+      }
+      if (__any_sync(full, open != 0)) {
+        const int wid = threadIdx.x >> 5;
+        if (open) {
+          uint32_t i = atomicAdd(&sh.n_open[wid], (uint32_t)__popc(open));
+#pragma unroll
+          for (int j = 0; j < kFastBatch; ++j)
+            if ((open >> j) & 1u) sh.open[wid][i++] = off[j];
+        }
+        __syncwarp();
+        if (sh.n_open[wid] >= kOpenRound) ops += drain_open(m, sh, kOpenRound);
       }
     }
-#pragma unroll
-    for (int j = 0; j < kFastBatchOf<kPipe>; ++j) {
-      if (((init >> j) & 1u) && __uint_as_float(old[j]) > m.l_min) {
-        atomicAdd(reinterpret_cast<float*>(occ + off[j]), m.miss);
-        ++ops;
-      }
-    }
-  };
-  if constexpr (kPipe) {
-    uint32_t offA[kFastBatchOf<kPipe>], offB[kFastBatchOf<kPipe>];
-    unsigned int oldA[kFastBatchOf<kPipe>], oldB[kFastBatchOf<kPipe>];
-    uint32_t vA = fill(offA), vB;
-    issue(offA, vA, oldA);
-    while (vA) {
-      vB = fill(offB);
-      issue(offB, vB, oldB);
-      apply(offA, vA, oldA);
-      if (!vB) break;
-      vA = fill(offA);
-      issue(offA, vA, oldA);
-      apply(offB, vB, oldB);
-    }
-  } else {
-    while (left > 0) {
-      uint32_t off[kFastBatchOf<kPipe>];
-      unsigned int old[kFastBatchOf<kPipe>];
-      const uint32_t v = fill(off);
-      issue(off, v, old);
-      apply(off, v, old);
-    }
+    K += kPieceSlots;
+    more = more && K < K1;
   }
 }
 
-// Whether a map's misses need the compare-and-swap form of walk_segment_fast.
+// Whether a map's misses need the compare-and-swap form of walk_segments.
 __device__ __host__ __forceinline__ bool walk_needs_cas(uint32_t layers, float miss, float ndt_clear) {
   return !(miss < 0.0f) || ((layers & kLayerNdt) && ndt_clear > -INFINITY);
 }
@@ -847,7 +985,14 @@ __device__ __forceinline__ void logodds_update_n(const DeviceMap& m, float* p, f
     const unsigned int nb = __float_as_uint(v);
     if (nb == old) return;
     const unsigned int prev = atomicCAS(u, old, nb);
-    if (prev == old) return;
+    if (prev == old) {
+      // a voxel stored at or below l_min may have its bit set
+      if (__uint_as_float(old) <= m.l_min) {
+        const long long off = p - m.occ;
+        atomicAnd(m.sat + (off >> 5), ~(1u << (off & 31)));
+      }
+      return;
+    }
     old = prev;
   }
   atomicOr(m.status, kStatusCasLimit);
