@@ -325,13 +325,13 @@ __global__ void __launch_bounds__(kBlock) k_ndt_backward(DeviceMap m, CallArgs a
           w[k] = g[k];
           any = any || w[k] != 0.f;
         }
-        const long long* mom = m.ndt + (long long)ns * 10 * kRegionVoxels + mo;
+        const long long* mom = ndt_moments(m, ns, mo);
         const double cnt = (double)mom[0];
         if (any && cnt > 0.0) {
           double dv[3];
 #pragma unroll
           for (int k = 0; k < 3; ++k)
-            dv[k] = (double)(qe[k] - (long long)v[k] * U) * cell - (double)mom[(long long)(1 + k) * kRegionVoxels] * cell / cnt;
+            dv[k] = (double)(qe[k] - (long long)v[k] * U) * cell - (double)mom[1 + k] * cell / cnt;
           // (G + G^T) d with G upper triangular from the packed xx xy xz yy yz zz
           const double Gs[3][3] = {{2.0 * w[3], w[4], w[5]}, {w[4], 2.0 * w[6], w[7]}, {w[5], w[7], 2.0 * w[8]}};
 #pragma unroll

@@ -151,31 +151,7 @@ __global__ void __launch_bounds__(kBlock) k_batch_ndt_alloc(const BatchDesc* des
   }
 }
 
-// Miss walk of the maps with the decay layer (walk_segment).
-__global__ void __launch_bounds__(kBlock, OHM_WALK_MIN_BLOCKS) k_batch_walk(const BatchDesc* desc, const BatchStep* step) {
-  chain_enter();
-  __shared__ BatchShared sh;
-  batch_stage(sh, desc, step, kSegments, kWalkDecay);
-  const long long total = sh.pref[sh.n_maps];
-  OHM_BATCH_STRIDE(g, total) {
-    const int mi = batch_find(sh, g);
-    const DeviceMap& m = sh.maps[mi];
-    const long long si = g - sh.pref[mi];
-    if (si >= (long long)m.calls->segments) continue;
-    unsigned int cas = 0;  // not attributed per map in a batched step
-    const bool occ = (m.layers & kLayerOcc) != 0, cnt = (m.layers & kLayerCounts) != 0;
-    if (occ && cnt)
-      walk_segment<true, true, true>(m, si, cas);
-    else if (occ)
-      walk_segment<true, false, true>(m, si, cas);
-    else if (cnt)
-      walk_segment<false, true, true>(m, si, cas);
-    else
-      walk_segment<false, false, true>(m, si, cas);
-  }
-}
-
-// Filtered miss walk of the maps whose walk is kVariant (walk_variant): one
+// Miss walk of the maps whose walk is kVariant (walk_variant): one
 // launch per variant present in the batch, so that each kernel holds only its
 // own update code (one kernel for every variant spills heavily).
 template <int kVariant>
@@ -186,19 +162,18 @@ __global__ void __launch_bounds__(kBlock, OHM_FAST_MIN_BLOCKS) k_batch_walk_fast
   batch_stage(sh, desc, step, kSegments, kVariant);
   const long long total = sh.pref[sh.n_maps];  // a multiple of 32: whole warps iterate together
   unsigned int ops = 0;  // not attributed per map in a batched step
-  if ((threadIdx.x & 31) == 0) ws.n_open[threadIdx.x >> 5] = 0;
-  __syncwarp();
+  walk_shared_init(ws);
   int last = -1;
   OHM_BATCH_STRIDE(g, total) {
     const int mi = batch_find(sh, g);
     const DeviceMap& m = sh.maps[mi];
-    if (kVariant == 4 || kVariant == 6) {  // the voxels in hand belong to the warp's last map
+    if ((kVariant & 4) && !(kVariant & 1)) {  // the voxels in hand belong to the warp's last map
       if (last >= 0 && mi != last) drain_open(sh.maps[last], ws, 1u);
       last = mi;
     }
     const long long si = g - sh.pref[mi];
     const bool has = si < (long long)m.calls->segments;
-    walk_segments<(kVariant & 4) != 0, (kVariant & 2) != 0, (kVariant & 1) != 0>(
+    walk_segments<(kVariant & 4) != 0, (kVariant & 2) != 0, (kVariant & 1) != 0, (kVariant & kWalkDecay) != 0>(
         m, has, has ? m.segs[si] : make_int2(0, 0), ws, ops);
   }
   if (last >= 0) drain_open(sh.maps[last], ws, 1u);
@@ -347,12 +322,10 @@ cudaError_t enqueue_step(ohm_batch* b, cudaStream_t s, int* count) {
   // oversubscribed grid-stride launches, like the single-map walk
   const int wgrid = grid * OHM_WALK_OVERSUBSCRIBE;
   const uint32_t wv = b->walk_variants;
-  if (wv & (1u << kWalkDecay)) launch_chained(k_batch_walk, wgrid, s, b->d_desc, b->d_step);
-  if (wv & (1u << 7)) launch_chained(k_batch_walk_fast<7>, wgrid, s, b->d_desc, b->d_step);
-  if (wv & (1u << 6)) launch_chained(k_batch_walk_fast<6>, wgrid, s, b->d_desc, b->d_step);
-  if (wv & (1u << 5)) launch_chained(k_batch_walk_fast<5>, wgrid, s, b->d_desc, b->d_step);
-  if (wv & (1u << 4)) launch_chained(k_batch_walk_fast<4>, wgrid, s, b->d_desc, b->d_step);
-  if (wv & (1u << 2)) launch_chained(k_batch_walk_fast<2>, wgrid, s, b->d_desc, b->d_step);
+#define OHM_WALK_CASE(v) \
+  if (wv & (1u << v)) launch_chained(k_batch_walk_fast<v>, wgrid, s, b->d_desc, b->d_step);
+  OHM_WALK_VARIANTS(OHM_WALK_CASE)
+#undef OHM_WALK_CASE
   n += __builtin_popcount(wv);
   if (b->any_occ || b->any_ndt || b->any_mean) {
     launch_chained(k_batch_hits, ray_grid, s, b->d_desc, b->d_step);

@@ -134,6 +134,7 @@ __global__ void k_reset_slots(DeviceMap m, const int32_t* slots, int n, const in
       if (m.tsdf) m.tsdf[off] = make_float2(0.f, 0.f);
       if (v == 0) m.ndt_slot[slots[r]] = -1;
     } else {
+      // 10 words of the block per thread, neighbouring threads side by side
       long long* base = m.ndt + (long long)ndt_blocks[r - n] * 10 * per + v;
 #pragma unroll
       for (int k = 0; k < 10; ++k) base[(long long)k * per] = 0;

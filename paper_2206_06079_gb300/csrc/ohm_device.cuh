@@ -159,7 +159,7 @@ struct DeviceMap {
   int32_t* ndt_count;
   int32_t max_ndt;
   int32_t* ndt_pending;          // [max_rays] sample rays whose region prepare could not give an NDT block
-  long long* ndt;                // [max_ndt][10][32768]
+  long long* ndt;                // [max_ndt][32768][10], a voxel's moments side by side (see ndt_moments)
   float2* tsdf;                  // [max_regions][32768] (D, W)
   uint32_t* tsdf_cnt;            // [max_regions][32768] per-call scratch, zero between calls
   long long* tsdf_sum;           // [max_regions][32768] per-call scratch, 2^-32 m units

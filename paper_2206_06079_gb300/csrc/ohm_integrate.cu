@@ -10,8 +10,8 @@
 //                    block of the sample's region
 //   k_ndt_alloc      sample rays prepare left: give their regions an NDT layer
 //   k_prepare_tsdf   per ray: TSDF band end points and their regions
-//   k_walk_fast      per segment: exact voxel walk, miss update per voxel
-//                    (k_walk_miss for maps with the decay layer)
+//   k_walk_fast      per segment: exact voxel walk, miss update per voxel,
+//                    counts and decay path lengths
 //   k_hits           per sample: hit update, hit count, NDT moments
 //   k_tsdf_walk      per ray: band walk, fixed-point s sums and counts
 //   k_tsdf_apply     per touched voxel: weighted average, scratch cleared
@@ -51,36 +51,25 @@ __global__ void __launch_bounds__(kBlock) k_ndt_alloc(DeviceMap m) {
   OHM_GRID_STRIDE(k, n) ndt_alloc_ray(m, m.ndt_pending[k]);
 }
 
-template <bool kOcc, bool kCounts, bool kDecay>
-__global__ void __launch_bounds__(kBlock, OHM_WALK_MIN_BLOCKS) k_walk_miss(DeviceMap m) {
-  chain_enter();
-  if (latched(m)) return;
-  const long long nseg = (long long)m.calls->segments;
-  unsigned int cas = 0;
-  OHM_GRID_STRIDE(si, nseg) walk_segment<kOcc, kCounts, kDecay>(m, si, cas);
-  // every thread gets here: one atomic per warp for the call's CAS count
-  cas = __reduce_add_sync(0xffffffffu, cas);
-  if ((threadIdx.x & 31) == 0 && cas) atomicAdd(&m.calls->atomics, (unsigned long long)cas);
-}
-
-// The miss walk of maps without the decay layer (walk_segments).
-template <bool kOcc, bool kCounts, bool kCas>
+// The miss walk (walk_segments); kVariant: walk_variant.
+template <int kVariant>
 __global__ void __launch_bounds__(kBlock, OHM_FAST_MIN_BLOCKS) k_walk_fast(DeviceMap m) {
+  constexpr bool kOcc = (kVariant & 4) != 0, kCounts = (kVariant & 2) != 0, kCas = (kVariant & 1) != 0;
+  constexpr bool kDecay = (kVariant & kWalkDecay) != 0;
   chain_enter();
   if (latched(m)) return;
   __shared__ WalkShared sh;
   const long long nseg = (long long)m.calls->segments;
   const long long stride = (long long)gridDim.x * kBlock;
   unsigned int ops = 0;
-  if ((threadIdx.x & 31) == 0) sh.n_open[threadIdx.x >> 5] = 0;
-  __syncwarp();
+  walk_shared_init(sh);
   long long si = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   int2 sg = si < nseg ? m.segs[si] : make_int2(0, 0);
   // whole warps iterate together
   for (; si - (threadIdx.x & 31) < nseg; si += stride) {
     // the next segment's table entry is loaded while this one walks
     const int2 next = si + stride < nseg ? m.segs[si + stride] : make_int2(-1, 0);
-    walk_segments<kOcc, kCounts, kCas>(m, si < nseg, sg, sh, ops, next.x >= 0 ? m.rays + next.x : nullptr);
+    walk_segments<kOcc, kCounts, kCas, kDecay>(m, si < nseg, sg, sh, ops, next.x >= 0 ? m.rays + next.x : nullptr);
     sg = next;
   }
   if (kOcc && !kCas) ops += drain_open(m, sh, 1u);
@@ -194,10 +183,14 @@ __global__ void __launch_bounds__(kBlock) k_query(DeviceMap m, const float* pts,
     for (int k = 0; k < 10; ++k) out[k] = 0.f;
     const int32_t ns = (slot >= 0 && (m.layers & kLayerNdt)) ? m.ndt_slot[slot] : -1;
     if (ns >= 0) {
-      const long long* base = m.ndt + (long long)ns * 10 * kRegionVoxels + mo;
+      const longlong2* base = reinterpret_cast<const longlong2*>(ndt_moments(m, ns, mo));
       long long s[10];
 #pragma unroll
-      for (int k = 0; k < 10; ++k) s[k] = base[(long long)k * kRegionVoxels];
+      for (int k = 0; k < 5; ++k) {
+        const longlong2 p = base[k];
+        s[2 * k] = p.x;
+        s[2 * k + 1] = p.y;
+      }
       if (s[0] > 0) {
         const double cnt = (double)s[0];
         const double cell = m.voxel_size / (double)(1LL << F);
@@ -220,36 +213,102 @@ __global__ void __launch_bounds__(kBlock) k_query(DeviceMap m, const float* pts,
   }
 }
 
-__global__ void __launch_bounds__(kBlock) k_export(DeviceMap m, long long first, long long count, int32_t* keys,
-                                                    float* occupancy, uint32_t* counts, long long* ndt, float* tsdf,
+// Two neighbouring elements of an exported row; in one store where the output
+// is aligned for it (kWide).
+template <bool kWide, typename T, typename T2>
+__device__ __forceinline__ void store_pair(T* out, T2 v) {
+  if (kWide) {
+    *reinterpret_cast<T2*>(out) = v;
+  } else {
+    out[0] = v.x;
+    out[1] = v.y;
+  }
+}
+
+// Export of regions in allocation order, voxels x fastest.  One block per slab
+// of two z layers of a region, one 2 x 2 x 2 brick of voxels per thread: in
+// Morton order a brick is contiguous (a sector of floats), so every layer is
+// read with whole 16-byte loads and written as four x pairs, 16 lanes side by
+// side filling a row.  NDT moments are copied row by row in 16-byte pieces,
+// five per voxel.  Bound by memory: a map of 192 regions with occupancy,
+// counts and NDT (1.16 GB moved) and a lookup took 429 us as one voxel per
+// thread, which read scattered floats and wrote 80-byte-strided words; this
+// form takes 205 us, 84 % of copy bandwidth.
+// kWide: every output pointer is 16-byte aligned.
+constexpr int kExportSlabs = 16;
+template <bool kWide>
+__global__ void __launch_bounds__(kBlock) k_export(DeviceMap m, long long first, int32_t* keys, float* occupancy,
+                                                    uint32_t* counts, long long* ndt, float* tsdf,
                                                     unsigned long long* path_sum, unsigned long long* mean) {
-  const long long total = count * kRegionVoxels;
-  for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    const long long r = t / kRegionVoxels;
-    const int32_t lin = (int32_t)(t % kRegionVoxels);
-    const int32_t slot = (int32_t)(first + r);
-    const uint32_t mo = morton(lin & 31, (lin >> 5) & 31, lin >> 10);
-    const long long off = voxel_offset(slot, mo);
-    if (keys && lin < 3) keys[3 * r + lin] = m.region_coords[3 * slot + lin];
-    if (occupancy) occupancy[t] = (m.layers & kLayerOcc) ? logodds_read(m.occ[off], m.l_min) : __int_as_float(0x7fc00000);
-    if (counts) {
-      const unsigned long long c = (m.layers & kLayerCounts) ? m.counts[off] : 0ULL;
-      counts[2 * t + 0] = (uint32_t)(c >> 32);
-      counts[2 * t + 1] = (uint32_t)(c & 0xffffffffu);
-    }
-    if (path_sum) path_sum[t] = (m.layers & kLayerDecay) ? m.decay[off] : 0ULL;
-    if (mean) mean[t] = (m.layers & kLayerMean) ? m.vmean[off] : 0ULL;
-    if (tsdf) {
-      const float2 dw = (m.layers & kLayerTsdf) ? m.tsdf[off] : make_float2(0.f, 0.f);
-      tsdf[2 * t + 0] = dw.x;
-      tsdf[2 * t + 1] = dw.y;
-    }
-    if (ndt) {
-      const int32_t ns = (m.layers & kLayerNdt) ? m.ndt_slot[slot] : -1;
+  const long long r = blockIdx.x / kExportSlabs;
+  const int slab = blockIdx.x % kExportSlabs, t = threadIdx.x;
+  const int32_t slot = (int32_t)(first + r);
+  if (keys && slab == 0 && t < 3) keys[3 * r + t] = m.region_coords[3 * slot + t];
+  const int x = 2 * (t & 15), y = 2 * (t >> 4), z = 2 * slab;
+  const long long off = voxel_offset(slot, morton(x, y, z));       // the brick's first voxel
+  const long long lin = r * kRegionVoxels + x + 32 * (y + 32 * z);  // and its place in the outputs
+  // rows of the brick: (y, z), (y + 1, z), (y, z + 1), (y + 1, z + 1)
+  const int row[4] = {0, 32, 1024, 1056};
+  if (occupancy) {
+    const float4* src = reinterpret_cast<const float4*>(m.occ + off);
+    const float4 a = src[0], b = src[1];
+    const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
 #pragma unroll
-      for (int k = 0; k < 10; ++k)
-        ndt[10 * t + k] = ns >= 0 ? m.ndt[(long long)ns * 10 * kRegionVoxels + (long long)k * kRegionVoxels + mo] : 0;
+    for (int k = 0; k < 4; ++k)
+      store_pair<kWide>(occupancy + lin + row[k],
+                        make_float2(logodds_read(v[2 * k], m.l_min), logodds_read(v[2 * k + 1], m.l_min)));
+  }
+  if (counts) {
+    const ulonglong2* src = reinterpret_cast<const ulonglong2*>(m.counts + off);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const ulonglong2 c = src[k];
+      uint32_t* o = counts + 2 * (lin + row[k]);
+      const uint4 v = make_uint4((uint32_t)(c.x >> 32), (uint32_t)c.x, (uint32_t)(c.y >> 32), (uint32_t)c.y);
+      if (kWide) {
+        *reinterpret_cast<uint4*>(o) = v;
+      } else {
+        o[0] = v.x;
+        o[1] = v.y;
+        o[2] = v.z;
+        o[3] = v.w;
+      }
+    }
+  }
+  auto words = [&](const unsigned long long* layer, unsigned long long* out) {
+    const ulonglong2* src = reinterpret_cast<const ulonglong2*>(layer + off);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) store_pair<kWide>(out + lin + row[k], src[k]);
+  };
+  if (path_sum) words(m.decay, path_sum);
+  if (mean) words(m.vmean, mean);
+  if (tsdf) {
+    const float4* src = reinterpret_cast<const float4*>(m.tsdf + off);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float4 v = src[k];
+      float* o = tsdf + 2 * (lin + row[k]);
+      if (kWide) {
+        *reinterpret_cast<float4*>(o) = v;
+      } else {
+        o[0] = v.x;
+        o[1] = v.y;
+        o[2] = v.z;
+        o[3] = v.w;
+      }
+    }
+  }
+  if (ndt) {
+    const int32_t ns = m.ndt_slot[slot];
+    longlong2* const out = reinterpret_cast<longlong2*>(ndt + (r * kRegionVoxels + 2048LL * slab) * 10);
+    // 64 rows of 32 voxels of 5 pieces
+#pragma unroll 8
+    for (int i = t; i < 64 * 160; i += kBlock) {
+      const int vox = i / 5, part = i - 5 * vox;
+      longlong2 v = make_longlong2(0, 0);
+      if (ns >= 0)
+        v = reinterpret_cast<const longlong2*>(ndt_moments(m, ns, morton(vox & 31, (vox >> 5) & 31, z + (vox >> 10))))[part];
+      store_pair<kWide>(reinterpret_cast<long long*>(out + i), v);
     }
   }
 }
@@ -259,7 +318,7 @@ __global__ void __launch_bounds__(kBlock) k_export(DeviceMap m, long long first,
 // ---------------------------------------------------------------------------
 int walk_blocks_per_sm() {
   int b = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_walk_fast<true, false, false>, kBlock, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_walk_fast<4>, kBlock, 0);
   return b > 0 ? b : 1;
 }
 
@@ -298,25 +357,12 @@ cudaError_t launch_integrate(ohm_map* map, const CallArgs& args, cudaStream_t st
     if (ndt) OHM_LAUNCH(OHM_STAGE_NDT_ALLOC, launch_chained(k_ndt_alloc, kNdtPendingGrid, stream, m));
   }
   if (tsdf) OHM_LAUNCH(OHM_STAGE_PREPARE_TSDF, launch_chained(k_prepare_tsdf, prb, stream, m, args));
-  const bool dec = (m.layers & kLayerDecay) != 0;
-  if (dec) {
-    const int sel = (occ ? 2 : 0) | (cnt ? 1 : 0);
-    switch (sel) {
-      case 3: OHM_LAUNCH(OHM_STAGE_WALK, launch_chained(k_walk_miss<true, true, true>, wgrid, stream, m)); break;
-      case 2: OHM_LAUNCH(OHM_STAGE_WALK, launch_chained(k_walk_miss<true, false, true>, wgrid, stream, m)); break;
-      case 1: OHM_LAUNCH(OHM_STAGE_WALK, launch_chained(k_walk_miss<false, true, true>, wgrid, stream, m)); break;
-      default: OHM_LAUNCH(OHM_STAGE_WALK, launch_chained(k_walk_miss<false, false, true>, wgrid, stream, m)); break;
-    }
-  } else if (occ || cnt) {
-    const bool c = walk_needs_cas(m.layers, m.miss, m.ndt_clear);
-    const int sel = (occ ? 4 : 0) | (cnt ? 2 : 0) | (c ? 1 : 0);
-    switch (sel) {
-      case 7: OHM_LAUNCH(OHM_STAGE_WALK, launch_chained(k_walk_fast<true, true, true>, wgrid, stream, m)); break;
-      case 6: OHM_LAUNCH(OHM_STAGE_WALK, launch_chained(k_walk_fast<true, true, false>, wgrid, stream, m)); break;
-      case 5: OHM_LAUNCH(OHM_STAGE_WALK, launch_chained(k_walk_fast<true, false, true>, wgrid, stream, m)); break;
-      case 4: OHM_LAUNCH(OHM_STAGE_WALK, launch_chained(k_walk_fast<true, false, false>, wgrid, stream, m)); break;
-      default: OHM_LAUNCH(OHM_STAGE_WALK, launch_chained(k_walk_fast<false, true, false>, wgrid, stream, m)); break;
-    }
+  switch (walk_variant(m.layers, m.miss, m.ndt_clear)) {
+#define OHM_WALK_CASE(v) \
+  case v: OHM_LAUNCH(OHM_STAGE_WALK, launch_chained(k_walk_fast<v>, wgrid, stream, m)); break;
+    OHM_WALK_VARIANTS(OHM_WALK_CASE)
+#undef OHM_WALK_CASE
+    default: break;  // kWalkNone
   }
   if (occ || cnt || ndt || mean) {
     const int sel = (occ ? 4 : 0) | (cnt ? 2 : 0) | (ndt ? 1 : 0);
@@ -491,10 +537,15 @@ cudaError_t launch_export(ohm_map* map, long long first, long long count, int32_
                           uint32_t* counts, long long* ndt, float* tsdf, unsigned long long* path_sum,
                           unsigned long long* mean, cudaStream_t stream) {
   if (count > 0) {
-    long long b = blocks_for(count * kRegionVoxels);
-    if (b > 65535LL * 16) b = 65535LL * 16;
-    k_export<<<(unsigned)b, kBlock, 0, stream>>>(map->d, first, count, keys, occupancy, counts, ndt, tsdf, path_sum,
-                                                  mean);
+    const unsigned blocks = (unsigned)(count * kExportSlabs);  // at most 2^20
+    uintptr_t low = 0;
+    for (const void* p : {(const void*)occupancy, (const void*)counts, (const void*)ndt, (const void*)tsdf,
+                          (const void*)path_sum, (const void*)mean})
+      low |= reinterpret_cast<uintptr_t>(p);
+    if (low & 15)
+      k_export<false><<<blocks, kBlock, 0, stream>>>(map->d, first, keys, occupancy, counts, ndt, tsdf, path_sum, mean);
+    else
+      k_export<true><<<blocks, kBlock, 0, stream>>>(map->d, first, keys, occupancy, counts, ndt, tsdf, path_sum, mean);
   }
   return cudaGetLastError();
 }

@@ -202,6 +202,14 @@ __device__ __forceinline__ int32_t region_slot_of(const DeviceMap& m, int32_t vx
 
 __device__ __forceinline__ uint32_t local_morton(int32_t vx, int32_t vy, int32_t vz) { return region_morton(vx, vy, vz); }
 
+// The 10 moments (n, Sx, Sy, Sz, Sxx, Sxy, Sxz, Syy, Syz, Szz) of a voxel of
+// NDT block ns.  They lie side by side, 80 bytes on a 16-byte boundary: a
+// sample, a query or an exported voxel touches 3 sectors instead of one in
+// each of 10 planes.
+__device__ __forceinline__ long long* ndt_moments(const DeviceMap& m, int32_t ns, uint32_t mo) {
+  return m.ndt + ((long long)ns * kRegionVoxels + mo) * 10;
+}
+
 // Sample clearing (Sec. II-D): a miss that took voxel `off` from at or above
 // the threshold (or from unknown) to below it clears the voxel's NDT samples.
 // Misses only lower a voxel within the miss phase, so exactly one successful
@@ -212,9 +220,9 @@ __device__ __forceinline__ void after_miss(const DeviceMap& m, long long off, un
   if (!(m.layers & kLayerNdt)) return;
   const int32_t ns = m.ndt_slot[off >> (3 * kRegionShift)];
   if (ns < 0) return;
-  long long* base = m.ndt + (long long)ns * 10 * kRegionVoxels + (off & (kRegionVoxels - 1));
+  long long* base = ndt_moments(m, ns, (uint32_t)off & (kRegionVoxels - 1));
 #pragma unroll
-  for (int k = 0; k < 10; ++k) base[(long long)k * kRegionVoxels] = 0;
+  for (int k = 0; k < 10; ++k) base[k] = 0;
 }
 
 // Retry a clamped log-odds CAS whose first attempt found `cur` instead of
@@ -250,20 +258,11 @@ __device__ __forceinline__ void miss_cas(const DeviceMap& m, unsigned int* u, un
 }
 
 // Launch shapes (measured on GB300, tunnel scans of 131,072 rays):
-//  OHM_WALK_BATCH          voxels in flight per thread in the miss walk
-//  OHM_WALK_MIN_BLOCKS     blocks of 256 threads per SM the walk is compiled for
-//                          (5: 48 registers; 4 and 6 were slower)
 //  OHM_WALK_OVERSUBSCRIBE  the walk's grid-stride launch covers this many
-//                          times the resident blocks
+//                          times the resident blocks (2, 4, 6, 8: 73.0, 72.4,
+//                          74.3, 75.4 us mapped, 179, 154, 156, 160 us unknown)
 //  OHM_PREPARE_MIN_BLOCKS  blocks per SM of the prepare kernels (4: a
 //                          131,072-ray scan fits one wave on 152 SMs)
-#ifndef OHM_WALK_BATCH
-#define OHM_WALK_BATCH 4
-#endif
-#ifndef OHM_WALK_MIN_BLOCKS
-#define OHM_WALK_MIN_BLOCKS 5
-#endif
-constexpr int kWalkBatch = OHM_WALK_BATCH;
 #ifndef OHM_WALK_OVERSUBSCRIBE
 #define OHM_WALK_OVERSUBSCRIBE 4
 #endif
@@ -458,118 +457,24 @@ __device__ __forceinline__ void ndt_alloc_ray(const DeviceMap& m, long long i) {
   ndt_claim(m, slot);
 }
 
-// Miss phase (Sec. III-C phase one) for one segment: every voxel a ray passes
-// through, except the voxel holding its sample, takes one miss.  Segment j of
-// a ray covers the voxels entered after j*S and before (j+1)*S steps of the
-// ray's dominant axis (the last segment runs to the end).
-//
-// The walk itself is cheap integer arithmetic; the cost is the read-modify-
-// write of each voxel in global memory.  So the thread walks kWalkBatch voxels
-// ahead, then issues all their loads at once, then all their CASes at once,
-// keeping that many memory operations in flight instead of one.
 // Decay layer: distance along the ray, in 2^-20 m, at which the walk crosses
 // a boundary of an axis that has taken `done` steps.  The crossing happens at
 // t = dist / A with dist = d0 + done U; t is taken as floor(2^32 dist / A) /
 // 2^32 (exact, by the reciprocal inv = reciprocal64(A); 2^32 dist < 2^62) and
 // the distance as rint(t L).  Monotone in t, so per-voxel differences are
 // never negative, and they add up to L over the ray.
-__device__ __forceinline__ unsigned long long decay_position(long long dist, int32_t A, unsigned long long inv,
+//
+// dist is below 2^31 (a ray is shorter than 2^30 units and U at most 2^20), so
+// the quotient's estimate floor(2^32 dist inv / 2^64) = floor(dist inv / 2^32)
+// takes two 32-bit multiplies; one remainder test makes it exact (div_by_inv).
+__device__ __forceinline__ unsigned long long decay_position(uint32_t dist, uint32_t A, unsigned long long inv,
                                                              unsigned long long length) {
-  const unsigned long long tq = div_by_inv((unsigned long long)dist << 32, (unsigned long long)A, inv);
+  unsigned long long tq = (unsigned long long)dist * (uint32_t)(inv >> 32) +
+                          (((unsigned long long)dist * (uint32_t)inv) >> 32);
+  if (((unsigned long long)dist << 32) - tq * A >= A) tq += 1;
   const unsigned long long lo = tq * length, hi = __umul64hi(tq, length);
   const unsigned long long lo2 = lo + (1ULL << 31);
   return ((hi + (lo2 < lo ? 1ULL : 0ULL)) << 32) | (lo2 >> 32);
-}
-
-template <bool kOcc, bool kCounts, bool kDecay>
-__device__ __forceinline__ void walk_segment(const DeviceMap& m, long long si, unsigned int& cas) {
-  const int F = m.frac_bits;
-  const int2 sg = m.segs[si];
-  const RayRec r = m.rays[sg.x];
-  const int M = (r.flags >> kRayAxisShift) & 3;
-  const bool last = sg.y == r.nseg - 1;
-  const bool sample = (r.flags & kRaySample) != 0;
-  long long K0, K1;
-  segment_bounds(M == 0 ? r.n[0] : (M == 1 ? r.n[1] : r.n[2]), r.nseg, (int32_t)((uint32_t)r.flags >> kRaySegShift),
-                 sg.y, &K0, &K1);
-  Walker w;
-  walker_init_rec(w, r, F, M, K0);
-  int32_t mrem = last ? INT_MAX : (int32_t)(K1 - K0 - 1);
-  int32_t slot = region_slot_of(m, w.vx, w.vy, w.vz);
-  if (slot < 0) {
-    atomicOr(m.status, kStatusMissing);
-    return;
-  }
-  uint32_t mo = local_morton(w.vx, w.vy, w.vz);
-  // decay layer: position (2^-20 m along the ray) where the walk entered the current voxel
-  DecayRec dr;
-  unsigned long long pos_in = 0;
-  if (kDecay) {
-    dr = m.decay_rays[sg.x];
-    if (K0 > 0) {
-      const int32_t d0M = M == 0 ? r.d0[0] : (M == 1 ? r.d0[1] : r.d0[2]);
-      const int32_t AM = M == 0 ? r.A[0] : (M == 1 ? r.A[1] : r.A[2]);
-      pos_in = decay_position((long long)d0M + ((K0 - 1) << F), AM, r.inv, dr.length);
-    }
-  }
-  bool done = false;
-  while (!done) {
-    uint32_t off[kWalkBatch];  // voxel offsets (< 2^31: at most 2^16 regions of 2^15 voxels)
-    uint32_t todo = 0;         // bit j: off[j] takes a miss
-#pragma unroll
-    for (int j = 0; j < kWalkBatch; ++j) {
-      off[j] = 0;
-      if (done) continue;
-      // the current voxel takes a miss unless it holds this ray's sample
-      off[j] = (uint32_t)voxel_offset(slot, mo);
-      if (!(sample && w.total == 0)) {
-        todo |= 1u << j;
-        if (kCounts) atomicAdd(m.counts + off[j], 1ULL);
-      }
-      if (w.total == 0) {
-        if (kDecay && dr.length != pos_in) atomicAdd(m.decay + off[j], dr.length - pos_in);
-        done = true;
-        continue;
-      }
-      const int axis = walker_choose(w);
-      if (kDecay) {
-        const int32_t d0a = axis == 0 ? r.d0[0] : (axis == 1 ? r.d0[1] : r.d0[2]);
-        const int32_t Aa = axis == 0 ? r.A[0] : (axis == 1 ? r.A[1] : r.A[2]);
-        const int32_t taken = axis == 0 ? r.n[0] - w.nx : (axis == 1 ? r.n[1] - w.ny : r.n[2] - w.nz);
-        const unsigned long long inv = axis == 0 ? dr.inv[0] : (axis == 1 ? dr.inv[1] : dr.inv[2]);
-        const unsigned long long pos_out = decay_position((long long)d0a + ((long long)taken << F), Aa, inv, dr.length);
-        const unsigned long long d = pos_out - pos_in;
-        if (d) atomicAdd(m.decay + off[j], d);
-        pos_in = pos_out;
-      }
-      if (axis == M) {
-        if (mrem == 0) {
-          done = true;
-          continue;
-        }
-        --mrem;
-      }
-      int32_t c, s;
-      walker_step(w, axis, &c, &s);
-      mo = morton_step(mo, morton_mask(axis), s);
-      if ((c & ((1 << kRegionShift) - 1)) == (s > 0 ? 0 : (1 << kRegionShift) - 1)) {
-        slot = region_slot_of(m, w.vx, w.vy, w.vz);
-        if (slot < 0) {
-          atomicOr(m.status, kStatusMissing);
-          done = true;
-        }
-      }
-    }
-    if (kOcc) {
-      unsigned int* base = reinterpret_cast<unsigned int*>(m.occ);
-      unsigned int old[kWalkBatch];
-#pragma unroll
-      for (int j = 0; j < kWalkBatch; ++j) old[j] = (todo >> j) & 1u ? base[off[j]] : 0u;
-#pragma unroll
-      for (int j = 0; j < kWalkBatch; ++j)
-        if ((todo >> j) & 1u) miss_cas(m, base + off[j], old[j], cas);
-    }
-  }
 }
 
 // Pool slots of two regions (or -1), their first probes issued together.
@@ -645,7 +550,13 @@ struct WalkShared {
   uint32_t tab[8 * kBlock];
   uint32_t open[kBlock / 32][kOpenCap];
   uint32_t n_open[kBlock / 32];
+  uint32_t sum[kBlock];  // decay layer: path length of the lanes in one voxel, at its lowest lane; zero between steps
 };
+__device__ __forceinline__ void walk_shared_init(WalkShared& sh) {
+  if ((threadIdx.x & 31) == 0) sh.n_open[threadIdx.x >> 5] = 0;
+  sh.sum[threadIdx.x] = 0;
+  __syncwarp();
+}
 constexpr uint32_t kNoRegion = 0x80000000u;
 __device__ __forceinline__ uint32_t region_entry(int32_t slot, uint32_t neg, uint32_t idx) {
   return ((uint32_t)slot << (3 * kRegionShift)) ^ neg ^ (idx << (3 * kRegionShift));
@@ -769,6 +680,15 @@ __device__ __forceinline__ unsigned int drain_open(const DeviceMap& m, WalkShare
 // l_min gets its bit there; the hits clear it; a stale clear bit only costs
 // the look.
 //
+// Counts and path lengths (kCounts, kDecay).  Every visit adds to these, and
+// all rays of a scan pass the voxels around the sensor: one 64-bit atomic per
+// visit queued at the few words there (a 65,344-ray scan with both layers took
+// 409 us, 106 us in this form).  The lanes of a warp that stand in the same voxel (neighbouring rays
+// at the same depth) form a group (__match_any_sync) whose lowest lane adds for
+// all of them; their path lengths are summed in shared memory.  The sums are
+// of integers, so grouping changes nothing.  kDecay: the voxel holding a
+// sample takes path length too.
+//
 // A batch is stepped without a branch; one that met a near-tie is stepped
 // again exactly.  What bounds the walk is instruction issue (46 M warp
 // instructions for 19.3 M visits of a 131,072-ray tunnel scan, 83 M before)
@@ -778,7 +698,7 @@ __device__ __forceinline__ unsigned int drain_open(const DeviceMap& m, WalkShare
 // Measured (131,072-ray tunnel scan, 0.1 m, 865 k segments): 123.5 -> 72.4 us in
 // a mapped tunnel, 164 -> 154 us in unknown space; 262,144 rays at 0.05 m
 // 308 -> 162 us; outdoor scans into half-known space 144 -> 104 us.
-template <bool kOcc, bool kCounts, bool kCas>
+template <bool kOcc, bool kCounts, bool kCas, bool kDecay>
 __device__ __forceinline__ void walk_segments(const DeviceMap& m, bool has, int2 sg, WalkShared& sh,
                                               unsigned int& ops, const RayRec* prefetch = nullptr) {
   constexpr uint32_t kAll = (1u << kFastBatch) - 1u;
@@ -790,12 +710,18 @@ __device__ __forceinline__ void walk_segments(const DeviceMap& m, bool has, int2
   unsigned int* const occ = reinterpret_cast<unsigned int*>(global_ptr(m.occ));
   const uint32_t* const sat = global_ptr(m.sat);
   unsigned long long* const counts = global_ptr(m.counts);
+  unsigned long long* const decay = global_ptr(m.decay);
+  // 32 lanes' path lengths through one voxel (at most sqrt(3) voxels each) add up in 32 bits
+  const bool small = m.voxel_size < 70.0;
   int32_t K = 0, K1 = -1;  // the piece's first dominant-axis step, the segment's end (not yet known)
   bool more = has;
   while (__any_sync(full, more)) {
     LWalker w = {};
     uint32_t mo = 0;
     int32_t left = 0;
+    bool to_end = false, sample = false;   // (decay) the piece ends the ray, at a sample
+    uint32_t c0 = 0, c1 = 0, c2 = 0;       // (decay) crossings taken per axis
+    unsigned long long pos = 0, len = 0;   // (decay) where the walk entered the voxel, the ray's length
     if (more) {
       const RayRec r = *rp;
       const int M = (r.flags >> kRayAxisShift) & 3;
@@ -811,7 +737,18 @@ __device__ __forceinline__ void walk_segments(const DeviceMap& m, bool has, int2
       const int32_t K0 = K, Ke = K + kPieceSlots < K1 ? K + kPieceSlots : K1;
       PieceStart p;
       piece_start(r, F, K0, Ke, Ke == nmaj + 1, &p, &w);
-      left = p.visits - ((Ke == nmaj + 1 && (r.flags & kRaySample)) ? 1 : 0);
+      to_end = Ke == nmaj + 1;
+      sample = to_end && (r.flags & kRaySample);
+      left = p.visits - ((sample && !kDecay) ? 1 : 0);
+      if (kDecay) {
+        c0 = (uint32_t)p.c[0];
+        c1 = (uint32_t)p.c[1];
+        c2 = (uint32_t)p.c[2];
+        len = m.decay_rays[sg.x].length;
+        if (K0 > 0)
+          pos = decay_position((uint32_t)(M == 0 ? r.d0[0] : (M == 1 ? r.d0[1] : r.d0[2])) + ((uint32_t)(K0 - 1) << F),
+                               (uint32_t)(M == 0 ? r.A[0] : (M == 1 ? r.A[1] : r.A[2])), r.inv, len);
+      }
       const uint32_t neg = morton_neg(r.flags);
       const int32_t signs = (r.flags >> kRaySignShift) & 7;
       mo = local_morton(p.v[0], p.v[1], p.v[2]) ^ neg;
@@ -895,10 +832,54 @@ __device__ __forceinline__ void walk_segments(const DeviceMap& m, bool has, int2
     for (; rounds > 0; --rounds) {
       uint32_t at[kFastBatch], off[kFastBatch], v[kFastBatch], valid;
       fill(at, off, valid);
-      if (kCounts) {
+      if (kCounts || kDecay) {
+        const int lane = threadIdx.x & 31;
+        uint32_t missed = valid;  // the voxels that take a miss
+        if (kDecay && sample && left <= 0 && valid) missed &= ~(1u << (31 - __clz(valid)));
 #pragma unroll
-        for (int j = 0; j < kFastBatch; ++j)
-          if ((valid >> j) & 1u) atomicAdd(counts + off[j], 1ULL);
+        for (int j = 0; j < kFastBatch; ++j) {
+          const bool in = (valid >> j) & 1u;
+          uint32_t d = 0;
+          unsigned long long wide = 0;
+          if (kDecay && in) {
+            // leave the voxel across the next boundary, or end in it
+            const uint32_t moved = at[j] ^ (j + 1 < kFastBatch ? at[j + 1] : mo);
+            const int axis = (moved & 0x9249u) ? 0 : ((moved & 0x12492u) ? 1 : 2);
+            unsigned long long out = len;
+            if (!(to_end && left <= 0 && !(valid >> (j + 1)))) {
+              const uint32_t c = axis == 0 ? c0 : (axis == 1 ? c1 : c2);
+              out = decay_position((uint32_t)rp->d0[axis] + (c << F), (uint32_t)rp->A[axis],
+                                   global_ptr(m.decay_rays)[sg.x].inv[axis], len);
+              c0 += axis == 0;
+              c1 += axis == 1;
+              c2 += axis == 2;
+            }
+            wide = out - pos;
+            d = (uint32_t)wide;
+            pos = out;
+          }
+          const unsigned grp = __match_any_sync(full, in ? off[j] : (kNoRegion | (uint32_t)lane));
+          const int lead = __ffs(grp) - 1;
+          if (kCounts) {
+            const unsigned n = __popc(grp & __ballot_sync(full, (missed >> j) & 1u));
+            if (in && lane == lead && n) atomicAdd(counts + off[j], (unsigned long long)n);
+          }
+          if (kDecay) {
+            if (small) {
+              uint32_t* const sum = sh.sum + (threadIdx.x & ~31u) + lead;
+              if (in && d) atomicAdd(sum, d);
+              __syncwarp();
+              if (in && lane == lead) {
+                if (*sum) atomicAdd(decay + off[j], (unsigned long long)*sum);
+                *sum = 0;
+              }
+              __syncwarp();
+            } else if (in && wide) {
+              atomicAdd(decay + off[j], wide);
+            }
+          }
+        }
+        if (kDecay) valid = missed;
       }
       if (!kOcc) continue;
       if (kCas) {
@@ -947,16 +928,17 @@ __device__ __host__ __forceinline__ bool walk_needs_cas(uint32_t layers, float m
   return !(miss < 0.0f) || ((layers & kLayerNdt) && ndt_clear > -INFINITY);
 }
 
-// Which miss walk a map takes: kWalkDecay (walk_segment, decay layer), else
-// the filtered walk's template arguments as bits (4: occupancy, 2: counts,
-// 1: every miss a compare-and-swap), or kWalkNone (no layer the walk updates).
+// Which miss walk a map takes: walk_segments' template arguments as bits (8:
+// decay, 4: occupancy, 2: counts, 1: every miss a compare-and-swap), or
+// kWalkNone (no layer the walk updates).
 constexpr int kWalkNone = -1;
 constexpr int kWalkDecay = 8;
+#define OHM_WALK_VARIANTS(X) X(2) X(4) X(5) X(6) X(7) X(8) X(10) X(12) X(13) X(14) X(15)
 __device__ __host__ __forceinline__ int walk_variant(uint32_t layers, float miss, float ndt_clear) {
   const bool occ = (layers & kLayerOcc) != 0, cnt = (layers & kLayerCounts) != 0;
-  if (layers & kLayerDecay) return kWalkDecay;
-  if (!occ && !cnt) return kWalkNone;
-  return (occ ? 4 : 0) | (cnt ? 2 : 0) | ((occ && walk_needs_cas(layers, miss, ndt_clear)) ? 1 : 0);
+  const bool decay = (layers & kLayerDecay) != 0;
+  if (!occ && !cnt && !decay) return kWalkNone;
+  return (decay ? kWalkDecay : 0) | (occ ? 4 : 0) | (cnt ? 2 : 0) | ((occ && walk_needs_cas(layers, miss, ndt_clear)) ? 1 : 0);
 }
 
 // Position of a sample inside its voxel (fixed-point offset 0 .. 2^F - 1) in
@@ -1065,10 +1047,10 @@ __device__ __forceinline__ void hit_ray(const DeviceMap& m, long long i, bool ac
     const long long px = b[0] - (long long)vx * U;
     const long long py = b[1] - (long long)vy * U;
     const long long pz = b[2] - (long long)vz * U;
-    unsigned long long* base = reinterpret_cast<unsigned long long*>(m.ndt) + (long long)ns * 10 * kRegionVoxels + mo;
+    unsigned long long* base = reinterpret_cast<unsigned long long*>(ndt_moments(m, ns, mo));
     const long long vals[10] = {1, px, py, pz, px * px, px * py, px * pz, py * py, py * pz, pz * pz};
 #pragma unroll
-    for (int k = 0; k < 10; ++k) atomicAdd(base + (long long)k * kRegionVoxels, (unsigned long long)vals[k]);
+    for (int k = 0; k < 10; ++k) atomicAdd(base + k, (unsigned long long)vals[k]);
   }
 }
 
