@@ -179,9 +179,13 @@ __global__ void __launch_bounds__(kBlock, OHM_FAST_MIN_BLOCKS) k_batch_walk_fast
   if (last >= 0) drain_open(sh.maps[last], ws, 1u);
 }
 
+// kNdt: some map of the batch has the NDT layer.  Its shared memory (23 KB)
+// and code stay out of the kernel of batches without.
+template <bool kNdt>
 __global__ void __launch_bounds__(kBlock) k_batch_hits(const BatchDesc* desc, const BatchStep* step) {
   chain_enter();
   __shared__ BatchShared sh;
+  __shared__ HitShared hs;
   batch_stage(sh, desc, step, kRaysPadded);
   const long long total = sh.pref[sh.n_maps];  // a multiple of 32: whole warps iterate together
   OHM_BATCH_STRIDE(g, total) {
@@ -191,15 +195,15 @@ __global__ void __launch_bounds__(kBlock) k_batch_hits(const BatchDesc* desc, co
     const bool a = i < step->n[mi] && !latched(m);
     const int sel = ((m.layers & kLayerOcc) ? 4 : 0) | ((m.layers & kLayerCounts) ? 2 : 0) | ((m.layers & kLayerNdt) ? 1 : 0);
     switch (sel) {
-      case 7: hit_ray<true, true, true>(m, i, a); break;
-      case 6: hit_ray<true, true, false>(m, i, a); break;
-      case 5: hit_ray<true, false, true>(m, i, a); break;
-      case 4: hit_ray<true, false, false>(m, i, a); break;
-      case 3: hit_ray<false, true, true>(m, i, a); break;
-      case 2: hit_ray<false, true, false>(m, i, a); break;
-      case 1: hit_ray<false, false, true>(m, i, a); break;
+      case 7: hit_ray<true, true, kNdt>(m, i, a, &hs); break;
+      case 6: hit_ray<true, true, false>(m, i, a, &hs); break;
+      case 5: hit_ray<true, false, kNdt>(m, i, a, &hs); break;
+      case 4: hit_ray<true, false, false>(m, i, a, &hs); break;
+      case 3: hit_ray<false, true, kNdt>(m, i, a, &hs); break;
+      case 2: hit_ray<false, true, false>(m, i, a, &hs); break;
+      case 1: hit_ray<false, false, kNdt>(m, i, a, &hs); break;
       default:
-        if (m.layers & kLayerMean) hit_ray<false, false, false>(m, i, a);
+        if (m.layers & kLayerMean) hit_ray<false, false, false>(m, i, a, &hs);
         break;
     }
   }
@@ -328,7 +332,10 @@ cudaError_t enqueue_step(ohm_batch* b, cudaStream_t s, int* count) {
 #undef OHM_WALK_CASE
   n += __builtin_popcount(wv);
   if (b->any_occ || b->any_ndt || b->any_mean) {
-    launch_chained(k_batch_hits, ray_grid, s, b->d_desc, b->d_step);
+    if (b->any_ndt)
+      launch_chained(k_batch_hits<true>, ray_grid, s, b->d_desc, b->d_step);
+    else
+      launch_chained(k_batch_hits<false>, ray_grid, s, b->d_desc, b->d_step);
     ++n;
   }
   if (b->any_mean) {
