@@ -107,14 +107,6 @@ __device__ __forceinline__ CallArgs batch_args(const BatchStep* step, int i) {
 #define OHM_BATCH_STRIDE(g, total) \
   for (long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x; g < (total); g += (long long)gridDim.x * blockDim.x)
 
-// Chained like the stage kernels after it (its launch overlaps the tail of the
-// previous step's last kernel).
-__global__ void k_batch_begin(const BatchDesc* desc, const BatchStep* step) {
-  chain_enter();
-  const int i = threadIdx.x;
-  if (blockIdx.x == 0 && i < desc->n_maps) begin_call(desc->maps[i], batch_args(step, i));
-}
-
 // One instantiation per pass (occupancy-like layers, or the TSDF band), so
 // that each kernel holds only its own per-ray code.
 template <bool kTsdf>
@@ -246,15 +238,17 @@ __global__ void __launch_bounds__(kBlock) k_batch_tsdf_apply(const BatchDesc* de
   }
 }
 
-// One group of blocks per map rolls back that map if its call failed.
+// One group of blocks per map rolls back that map if its call failed, and
+// makes its counters ready for the next call.
 __global__ void k_batch_end(const BatchDesc* desc) {
   chain_enter();
   const int per_map = gridDim.x / kMaxBatchMaps;
   const int mi = blockIdx.x / per_map;
   if (mi >= desc->n_maps) return;
   const DeviceMap& m = desc->maps[mi];
-  if (!latched(m)) return;
   const long long b = blockIdx.x % per_map;
+  if (b == 0 && threadIdx.x == 0) finish_call(m);
+  if (!latched(m)) return;
   rollback_call(m, b * blockDim.x + threadIdx.x, (long long)per_map * blockDim.x);
 }
 
@@ -309,8 +303,7 @@ cudaError_t enqueue_step(ohm_batch* b, cudaStream_t s, int* count) {
   using namespace ohm;
   const int grid = b->num_sms * b->walk_blocks_per_sm;
   const int ray_grid = b->num_sms * 4;
-  launch_chained(k_batch_begin, 1, s, b->d_desc, b->d_step);
-  int n = 1;
+  int n = 0;
   if (b->any_occ || b->any_ndt || b->any_mean) {
     launch_chained(k_batch_prepare<false>, ray_grid, s, b->d_desc, b->d_step);
     ++n;
@@ -495,7 +488,10 @@ ohm_status ohm_batch_integrate(ohm_batch* b, const float* const* origins, const 
     }
   }
   if (e != cudaSuccess) return bfail(OHM_ERR_CUDA, std::string("batch_integrate: ") + cudaGetErrorString(e));
-  for (int i = 0; i < b->n_maps; ++i) ohm::note_work(b->maps[i], s);
+  for (int i = 0; i < b->n_maps; ++i) {
+    b->maps[i]->last_rays = n[i];
+    ohm::note_work(b->maps[i], s);
+  }
   return OHM_OK;
 }
 

@@ -203,6 +203,8 @@ cudaError_t write_pool(ohm_map* m, const PoolView& v) {
   if (e == cudaSuccess) e = cudaMemcpy(d.free_info, info, sizeof(info), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(d.region_count, &v.region_count, sizeof(int32_t), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(d.ndt_count, &v.ndt_count, sizeof(int32_t), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = launch_snapshot(m, 0);
+  if (e == cudaSuccess) e = cudaDeviceSynchronize();
   return e;
 }
 
@@ -399,7 +401,7 @@ cudaError_t cache_pending(ohm_map* m, std::vector<long long>* keys) {
   CallCounters c;
   cudaError_t e = cudaMemcpy(&c, m->d.calls, sizeof(c), cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return e;
-  const long long n = std::min<long long>((long long)c.restores, m->d.max_restore);
+  const long long n = std::min<long long>((long long)c.last.restores, m->d.max_restore);
   return d2h(*keys, m->d.restore_keys, (size_t)n);
 }
 

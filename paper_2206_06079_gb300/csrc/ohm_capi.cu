@@ -297,6 +297,12 @@ ohm_status ohm_map_create(const ohm_map_params* params, ohm_map** out) {
   if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&m->h_status), sizeof(int32_t));
   if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&m->h_calls), sizeof(ohm::CallCounters));
   if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&m->h_count), 2 * sizeof(int32_t));
+  if (e == cudaSuccess) {
+    // ready for the first call (number 1; nothing is born in call 0)
+    std::memset(m->h_calls, 0, sizeof(ohm::CallCounters));
+    m->h_calls->seq = 1;
+    e = cudaMemcpy(d.calls, m->h_calls, sizeof(ohm::CallCounters), cudaMemcpyHostToDevice);
+  }
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) {
     free_map(m);
@@ -573,15 +579,15 @@ ohm_status ohm_map_stats(ohm_map* map, ohm_call_stats* out, void* stream) {
     e = cudaMemcpyAsync(map->h_count + 1, map->d.ndt_count, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(e, "stats");
-  out->rays = (int64_t)map->h_calls->rays;
-  out->segments = (int64_t)map->h_calls->segments;
-  out->visits = (int64_t)map->h_calls->visits;
-  out->touched = (int64_t)map->h_calls->touched;
+  out->rays = (int64_t)map->last_rays;
+  out->segments = (int64_t)map->h_calls->last.segments;
+  out->visits = (int64_t)map->h_calls->last.visits;
+  out->touched = (int64_t)map->h_calls->last.touched;
   out->regions = map->h_count[0] < map->p.max_regions ? map->h_count[0] : map->p.max_regions;
   out->ndt_regions = map->h_count[1];
   out->total_visits = (int64_t)map->h_calls->total_visits;
   out->launches = map->launches;
-  out->atomics = (int64_t)map->h_calls->atomics;
+  out->atomics = (int64_t)map->h_calls->last.atomics;
   return OHM_OK;
 }
 

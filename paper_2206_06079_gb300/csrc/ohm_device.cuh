@@ -117,24 +117,25 @@ struct BandConsts {
   FF tau, rmin, rmax;  // fixed-point units
 };
 
+// Between calls they stand ready for the next one: k_end moves the finished
+// call's values to `last`, zeroes them and takes the pool snapshot.
 struct CallCounters {
   unsigned long long segments;
   unsigned long long visits;
   unsigned long long touched;
-  int32_t region_start;   // pool counters when the call began (rollback point)
-  int32_t ndt_start;
-  unsigned long long rays;
-  unsigned long long total_visits;  // every call since the map was made
-  int32_t seq;                      // sequence number of the current call (LRU stamps, birth marks)
-  int32_t free_used_start;          // free-list positions when the call began (rollback point)
-  int32_t ndt_free_used_start;
-  int32_t mean_touched;             // entries of mean_list written by the current call
-  unsigned long long restores;      // evicted region keys this call asked to restore
-  long long origin_q[3];            // the call's shared sensor origin, quantised (one origin only)
-  int32_t origin_ok;                // 1 if origin_q is valid
-  int32_t pad2;
-  unsigned long long atomics;       // log-odds CAS operations the miss walk issued (single-map calls)
+  unsigned long long atomics;       // log-odds atomics the miss walk issued (single-map calls)
   unsigned long long ndt_pending;   // entries of DeviceMap::ndt_pending written by the current call
+  unsigned long long restores;      // evicted region keys this call asked to restore
+  int32_t mean_touched;             // entries of mean_list written by the current call
+  int32_t seq;                      // sequence number of the current (or next) call (LRU stamps, birth marks)
+  int32_t region_start;             // pool counters before the call (rollback point)
+  int32_t ndt_start;
+  int32_t free_used_start;          // free-list positions before the call (rollback point)
+  int32_t ndt_free_used_start;
+  unsigned long long total_visits;  // every call since the map was made
+  struct {
+    unsigned long long segments, visits, touched, atomics, restores;
+  } last;                           // of the last finished call
 };
 
 // Everything a kernel needs, passed by value.
@@ -1098,7 +1099,6 @@ __device__ __forceinline__ unsigned long long warp_reserve(unsigned long long* c
   return base + incl - count;
 }
 
-// Warp sum of a 32-bit value, added by one lane to two 64-bit counters; full warp.
 // ---------------------------------------------------------------------------
 // TSDF band of a ray (Sec. II-F) from the double length len of its fixed-point
 // difference d (ray_length) and the band half-width tau (fixed-point units):
@@ -1401,12 +1401,10 @@ OHM_UNROLL
   return true;
 }
 
-__device__ __forceinline__ void warp_add(unsigned long long* counter, unsigned long long* counter2, unsigned int value) {
+// Warp sum of a 32-bit value, added by one lane to a 64-bit counter; full warp.
+__device__ __forceinline__ void warp_add(unsigned long long* counter, unsigned int value) {
   unsigned int total = __reduce_add_sync(0xffffffffu, value);
-  if ((threadIdx.x & 31) == 0 && total != 0) {
-    atomicAdd(counter, (unsigned long long)total);
-    atomicAdd(counter2, (unsigned long long)total);
-  }
+  if ((threadIdx.x & 31) == 0 && total != 0) atomicAdd(counter, (unsigned long long)total);
 }
 
 }  // namespace ohm

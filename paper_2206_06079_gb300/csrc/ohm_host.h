@@ -40,6 +40,7 @@ struct ohm_map {
   ohm::CallCounters* h_calls;
   int32_t* h_count;
   long long launches;       // kernels launched by this map
+  long long last_rays;      // rays of the last integrate call
   // per-stage event timing
   uint32_t profile_mask;
   int32_t profile_every;    // record only every profile_every-th call (0 or 1: every call)
@@ -70,6 +71,8 @@ cudaError_t launch_export(ohm_map* map, long long first, long long count, int32_
                           uint32_t* counts, long long* ndt, float* tsdf, unsigned long long* path_sum,
                           unsigned long long* mean, cudaStream_t stream);
 int walk_blocks_per_sm();
+// Take the rollback point again, after the pool counters were written between calls.
+cudaError_t launch_snapshot(ohm_map* map, cudaStream_t stream);
 
 // Region cache (ohm_cache.cu).
 cudaError_t cache_evict(ohm_map* m, long long target, long long* evicted);

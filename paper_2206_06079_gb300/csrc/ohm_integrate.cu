@@ -2,7 +2,6 @@
 // for sm_103a).
 //
 // One integrate call is one "ray set".  Kernels, in stream order:
-//   k_begin          snapshot the pool counters (the rollback point)
 //   k_prepare_occ    per ray: fixed-point quantisation, max-range truncation,
 //                    region walk with hash insertion (the paper does this on
 //                    the CPU, Sec. III-B; here it is a device pass), the
@@ -15,8 +14,9 @@
 //   k_hits           per sample: hit update, hit count, NDT moments
 //   k_tsdf_walk      per ray: band walk, fixed-point s sums and counts
 //   k_tsdf_apply     per touched voxel: weighted average, scratch cleared
-//   k_end            if any kernel latched a failure: undo the allocations
-// Every kernel after k_begin returns at once when the status word is set, so
+//   k_end            if any kernel latched a failure: undo the allocations;
+//                    counters and rollback point made ready for the next call
+// Every kernel returns at once when the status word is set, so
 // a failed call changes no voxel.
 #include "ohm_kernels.cuh"
 
@@ -24,13 +24,6 @@ namespace ohm {
 
 #define OHM_GRID_STRIDE(i, n) \
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < (n); i += (long long)gridDim.x * blockDim.x)
-
-// Chained like the kernels after it: its launch overlaps the tail of the
-// previous call's last kernel, and its body waits for that kernel.
-__global__ void k_begin(DeviceMap m, CallArgs args) {
-  chain_enter();
-  if (blockIdx.x == 0 && threadIdx.x == 0) begin_call(m, args);
-}
 
 __global__ void __launch_bounds__(kBlock, OHM_PREPARE_MIN_BLOCKS) k_prepare_occ(DeviceMap m, CallArgs args) {
   chain_enter();
@@ -120,9 +113,13 @@ __global__ void __launch_bounds__(kBlock) k_tsdf_apply(DeviceMap m) {
 
 __global__ void k_end(DeviceMap m) {
   chain_enter();
+  if (blockIdx.x == 0 && threadIdx.x == 0) finish_call(m);
   if (!latched(m)) return;
   rollback_call(m, (long long)blockIdx.x * blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
 }
+
+// The pool counters changed between calls (region cache).
+__global__ void k_snapshot(DeviceMap m) { snapshot_pool(m); }
 
 // ---------------------------------------------------------------------------
 // Query and export.
@@ -352,7 +349,7 @@ cudaError_t launch_integrate(ohm_map* map, const CallArgs& args, cudaStream_t st
   const long long per_ray_blocks = blocks_for(n) > 0 ? blocks_for(n) : 1;
   const int ray_grid = (int)(per_ray_blocks < grid ? per_ray_blocks : grid);
   const unsigned prb = (unsigned)per_ray_blocks;
-  OHM_LAUNCH(OHM_STAGE_BEGIN, launch_chained(k_begin, 1, stream, m, args));
+  map->last_rays = n;
   if (occ_like) {
     OHM_LAUNCH(OHM_STAGE_PREPARE, launch_chained(k_prepare_occ, prb, stream, m, args));
     if (ndt) OHM_LAUNCH(OHM_STAGE_NDT_ALLOC, launch_chained(k_ndt_alloc, kNdtPendingGrid, stream, m));
@@ -523,6 +520,11 @@ cudaError_t probe_rate(int device, int kind, long long units, long long ops, dou
   if (e1) cudaEventDestroy(e1);
   cudaFree(buf);
   return e;
+}
+
+cudaError_t launch_snapshot(ohm_map* map, cudaStream_t stream) {
+  k_snapshot<<<1, 1, 0, stream>>>(map->d);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_query(ohm_map* map, const float* points, long long n, float* occupancy, uint8_t* known, float* ndt,

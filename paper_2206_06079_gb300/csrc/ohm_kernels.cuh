@@ -280,46 +280,70 @@ __device__ __forceinline__ void miss_cas(const DeviceMap& m, unsigned int* u, un
 #define OHM_PREPARE_MIN_BLOCKS 4
 #endif
 
-// Snapshot of the pool counters at the start of a call (the rollback point).
-__device__ __forceinline__ void begin_call(const DeviceMap& m, const CallArgs& a) {
-  const long long n = a.n;
+// The rollback point of the next call: the pool counters as they stand.
+__device__ __forceinline__ void snapshot_pool(const DeviceMap& m) {
   m.calls->region_start = *m.region_count;
   m.calls->ndt_start = *m.ndt_count;
   m.calls->free_used_start = m.free_info[1];
   m.calls->ndt_free_used_start = m.free_info[3];
-  m.calls->seq += 1;
-  m.calls->segments = 0;
-  m.calls->visits = 0;
-  m.calls->touched = 0;
-  m.calls->mean_touched = 0;
-  m.calls->restores = 0;
-  m.calls->atomics = 0;
-  m.calls->ndt_pending = 0;
-  m.calls->rays = (unsigned long long)n;
-  // a shared sensor origin is quantised once for the whole call
-  bool ok = false;
-  if (a.n_origins == 1 && n > 0) {
-    ok = true;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const float o = a.origins[k];
-      long long q = 0;
-      ok = ok && isfinite(o) && quantise(o, m.origin[k], m.scale, &q);
-      m.calls->origin_q[k] = q;
-    }
+}
+
+// End of a call, one thread of its last kernel: its counters become `last`
+// and stand ready for the next call.  A failed call keeps its sequence number
+// and its rollback point, which the rollback (running beside this) reads.
+// Doing this here saves a kernel at the start of every call, about 3 us of a
+// small scan and one launch.
+__device__ __forceinline__ void finish_call(const DeviceMap& m) {
+  CallCounters* c = m.calls;
+  c->last.segments = c->segments;
+  c->last.visits = c->visits;
+  c->last.touched = c->touched;
+  c->last.atomics = c->atomics;
+  c->last.restores = c->restores;
+  c->total_visits += c->visits;
+  c->segments = 0;
+  c->visits = 0;
+  c->touched = 0;
+  c->atomics = 0;
+  c->restores = 0;
+  c->ndt_pending = 0;
+  c->mean_touched = 0;
+  if (!latched(m)) {
+    c->seq += 1;
+    snapshot_pool(m);
   }
-  m.calls->origin_ok = ok ? 1 : 0;
+}
+
+// Fixed-point origin of the current call's rays where they share one: the
+// first three lanes quantise a coordinate each.  Whole warps.
+struct CallOrigin {
+  long long q[3];
+  bool ok;
+};
+__device__ __forceinline__ CallOrigin call_origin(const DeviceMap& m, const CallArgs& a) {
+  const unsigned full = 0xffffffffu;
+  CallOrigin r = {{0, 0, 0}, false};
+  if (a.n_origins != 1 || a.n <= 0) return r;
+  const int lane = threadIdx.x & 31, k = lane < 3 ? lane : 2;
+  const float o = a.origins[k];
+  long long q = 0;
+  const bool ok = isfinite(o) && quantise(o, k == 0 ? m.origin[0] : (k == 1 ? m.origin[1] : m.origin[2]), m.scale, &q);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) r.q[i] = __shfl_sync(full, q, i);
+  r.ok = __all_sync(full, ok);
+  return r;
 }
 
 // quantise_ray for the rays of the current call: a shared origin comes
-// quantised from begin_call.
-__device__ __forceinline__ bool quantise_call_ray(const DeviceMap& m, const CallArgs& a, const float o[3],
-                                                  const float e[3], long long qo[3], long long qe[3]) {
+// quantised from call_origin.
+__device__ __forceinline__ bool quantise_call_ray(const DeviceMap& m, const CallArgs& a, const CallOrigin& origin,
+                                                  const float o[3], const float e[3], long long qo[3],
+                                                  long long qe[3]) {
   if (a.n_origins != 1) return quantise_ray(m, o, e, qo, qe);
-  bool ok = m.calls->origin_ok != 0;
+  bool ok = origin.ok;
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    qo[k] = m.calls->origin_q[k];
+    qo[k] = origin.q[k];
     ok = ok && isfinite(e[k]) && quantise(e[k], m.origin[k], m.scale, &qe[k]);
   }
   return ok;
@@ -359,6 +383,7 @@ __device__ __forceinline__ void write_segments(const DeviceMap& m, long long i, 
 // lanes without a ray pass active = false.
 __device__ __forceinline__ void prepare_occ_ray(const DeviceMap& m, const CallArgs& args, long long i, bool active) {
   active = active && !latched(m);
+  const CallOrigin origin = call_origin(m, args);
   const int F = m.frac_bits;
   unsigned int nseg = 0, nvisit = 0;
   bool ndt_listed = false;
@@ -371,7 +396,7 @@ __device__ __forceinline__ void prepare_occ_ray(const DeviceMap& m, const CallAr
     uint8_t flag;
     load_ray(args, i, o, e, &flag);
     long long qo[3], qe[3];
-    bool ok = quantise_call_ray(m, args, o, e, qo, qe);
+    bool ok = quantise_call_ray(m, args, origin, o, e, qo, qe);
     bool sample = (flag & kFlagNoReturn) == 0;
     if (ok) {
       // Truncation test len > rmax_q with len the double length: settled by
@@ -449,7 +474,7 @@ __device__ __forceinline__ void prepare_occ_ray(const DeviceMap& m, const CallAr
     }
   }
   write_segments(m, i, nseg);
-  warp_add(&m.calls->visits, &m.calls->total_visits, nvisit);
+  warp_add(&m.calls->visits, nvisit);
 }
 
 // Per sample: give the sample's region an NDT layer.
@@ -1073,6 +1098,7 @@ __device__ __forceinline__ void hit_ray(const DeviceMap& m, long long i, bool ac
 // quantised like a truncated endpoint.  Full warp, like prepare_occ_ray.
 __device__ __forceinline__ void prepare_tsdf_ray(const DeviceMap& m, const CallArgs& args, long long i, bool active) {
   active = active && !latched(m);
+  const CallOrigin origin = call_origin(m, args);
   const int F = m.frac_bits;
   unsigned int nvisit = 0;
   TsdfRec r;
@@ -1082,7 +1108,7 @@ __device__ __forceinline__ void prepare_tsdf_ray(const DeviceMap& m, const CallA
     uint8_t flag;
     load_ray(args, i, o, e, &flag);
     long long qo[3], qe[3];
-    bool ok = quantise_call_ray(m, args, o, e, qo, qe) && (flag & kFlagNoReturn) == 0;
+    bool ok = quantise_call_ray(m, args, origin, o, e, qo, qe) && (flag & kFlagNoReturn) == 0;
     if (ok) {
       // the range test and the band in float-float; in double where that
       // cannot settle them (tsdf_band_ff)
@@ -1110,7 +1136,7 @@ __device__ __forceinline__ void prepare_tsdf_ray(const DeviceMap& m, const CallA
     }
     m.trays[i] = r;
   }
-  warp_add(&m.calls->visits, &m.calls->total_visits, nvisit);
+  warp_add(&m.calls->visits, nvisit);
 }
 
 // TSDF band walk of one ray: per visited voxel c, s = (e - c).u (equal to
