@@ -619,6 +619,7 @@ ohm_status ohm_ndt_backward(ohm_map* map, const double* pose, const float* origi
     k_ndt_grad_scatter<<<qb, kBlock, 0, s>>>(map->d, query_points, grad_mean, grad_cov, n_query, 0);
     map->launches += 1;
   }
+  map->status_copied = false;  // k_ndt_backward can latch a failure
   if (e == cudaSuccess && n > 0) {
     CallArgs a;
     e = stage_posed(map, P, origins, n_origins, endpoints, flags, n, s, &a);

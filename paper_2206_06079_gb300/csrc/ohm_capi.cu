@@ -35,27 +35,26 @@ struct DeviceGuard {
   }
 };
 
-bool is_device_pointer(const void* p) {
-  if (!p) return false;
+// Where a pointer's memory is, from one lookup: device memory (or managed), and
+// device memory of another GPU than `dev` (the map's), which is rejected rather
+// than reached through peer access.  NULL is neither.
+struct Where {
+  bool device = false, other = false;
+};
+Where where_is(const void* p, int dev) {
+  Where w;
+  if (!p) return w;
   cudaPointerAttributes a;
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
     cudaGetLastError();
-    return false;
+    return w;
   }
-  return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
+  w.device = a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
+  w.other = a.type == cudaMemoryTypeDevice && a.device != dev;
+  return w;
 }
 
-// Device memory of another GPU than `dev` (the map's): rejected rather than
-// reached through peer access.
-bool on_other_device(const void* p, int dev) {
-  if (!p) return false;
-  cudaPointerAttributes a;
-  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  return a.type == cudaMemoryTypeDevice && a.device != dev;
-}
+bool is_device_pointer(const void* p) { return where_is(p, 0).device; }
 
 template <typename T>
 cudaError_t alloc(T** p, size_t count, int fill) {
@@ -130,11 +129,11 @@ ohm_status enqueue_integrate(ohm_map* map, const float* origins, int64_t n_origi
   a.origins = origins;
   a.endpoints = endpoints;
   a.flags = flags;
-  if (on_other_device(origins, map->device) || on_other_device(endpoints, map->device) ||
-      on_other_device(flags, map->device))
+  const Where wo = where_is(origins, map->device), we = where_is(endpoints, map->device);
+  const Where wf = where_is(flags, map->device);
+  if (wo.other || we.other || wf.other)
     return fail(OHM_ERR_INVALID, "integrate: inputs are on another device than the map");
-  const bool host_o = !is_device_pointer(origins), host_e = !is_device_pointer(endpoints);
-  const bool host_f = flags && !is_device_pointer(flags);
+  const bool host_o = !wo.device, host_e = !we.device, host_f = flags && !wf.device;
   cudaError_t e = cudaSuccess;
   int slot = -1;
   if (host_o || host_e || host_f) {
@@ -294,11 +293,13 @@ ohm_status ohm_map_create(const ohm_map_params* params, ohm_map** out) {
   }
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&m->copy_stream, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m->work_done, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&m->h_status), sizeof(int32_t));
+  if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&m->h_status), 2 * sizeof(int32_t));
   if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&m->h_calls), sizeof(ohm::CallCounters));
   if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&m->h_count), 2 * sizeof(int32_t));
   if (e == cudaSuccess) {
     // ready for the first call (number 1; nothing is born in call 0)
+    m->h_status[0] = m->h_status[1] = 0;
+    d.host_status = m->h_status + 1;  // pinned memory is mapped at the same address
     std::memset(m->h_calls, 0, sizeof(ohm::CallCounters));
     m->h_calls->seq = 1;
     e = cudaMemcpy(d.calls, m->h_calls, sizeof(ohm::CallCounters), cudaMemcpyHostToDevice);
@@ -359,11 +360,17 @@ ohm_status ohm_map_sync(ohm_map* map, void* stream) {
   if (!map) return fail(OHM_ERR_INVALID, "sync: map is NULL");
   DeviceGuard guard(map->device);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  cudaError_t e = cudaMemcpyAsync(map->h_status, map->d.status, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
+  // The last kernel of every integrate call writes the status to pinned host
+  // memory; only after other work that can latch one is the word copied (a
+  // copy on the stream takes about 4 us of a call that waits).
+  const bool copy = !map->status_copied;
+  cudaError_t e = cudaSuccess;
+  if (copy) e = cudaMemcpyAsync(map->h_status, map->d.status, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(e, "sync");
-  const int bits = *map->h_status;
+  const int bits = *(volatile int32_t*)(map->h_status + (copy ? 0 : 1));
   if (bits != 0) {
+    *(volatile int32_t*)(map->h_status + 1) = 0;
     e = cudaMemsetAsync(map->d.status, 0, sizeof(int32_t), s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(e, "sync: clear status");
@@ -504,9 +511,11 @@ ohm_status ohm_query_voxels(ohm_map* map, const float* points, int64_t n, float*
   if (n == 0) return OHM_OK;
   if (!points) return fail(OHM_ERR_INVALID, "query: points is NULL");
   void* outs[] = {occupancy, known, ndt, tsdf, counts, path_sum, mean};
-  for (void* o : outs)
-    if (o && (!is_device_pointer(o) || on_other_device(o, map->device)))
+  for (void* o : outs) {
+    const Where w = where_is(o, map->device);
+    if (o && (!w.device || w.other))
       return fail(OHM_ERR_INVALID, "query: outputs must be device memory of the map's device");
+  }
   if (path_sum && !(map->p.layers & OHM_LAYER_DECAY)) return fail(OHM_ERR_UNSUPPORTED, "query: map has no decay layer");
   if (mean && !(map->p.layers & OHM_LAYER_MEAN)) return fail(OHM_ERR_UNSUPPORTED, "query: map has no mean layer");
   if (ndt && !(map->p.layers & OHM_LAYER_NDT)) return fail(OHM_ERR_UNSUPPORTED, "query: map has no NDT layer");
@@ -516,8 +525,9 @@ ohm_status ohm_query_voxels(ohm_map* map, const float* points, int64_t n, float*
   const float* pts = points;
   float* staged = nullptr;
   cudaError_t e;
-  if (on_other_device(points, map->device)) return fail(OHM_ERR_INVALID, "query: points on another device than the map");
-  if (!is_device_pointer(points)) {
+  const Where wp = where_is(points, map->device);
+  if (wp.other) return fail(OHM_ERR_INVALID, "query: points on another device than the map");
+  if (!wp.device) {
     e = cudaMallocAsync(reinterpret_cast<void**>(&staged), sizeof(float) * 3 * n, s);
     if (e != cudaSuccess) return cuda_fail(e, "query: staging");
     e = cudaMemcpyAsync(staged, points, sizeof(float) * 3 * n, cudaMemcpyHostToDevice, s);
@@ -551,9 +561,11 @@ ohm_status ohm_map_export(ohm_map* map, int64_t first, int64_t count, int32_t* k
   if (first < 0 || count < 0 || first + count > map->p.max_regions)
     return fail(OHM_ERR_INVALID, "export: region range outside the pool");
   void* outs[] = {keys, occupancy, counts, ndt, tsdf, path_sum, mean};
-  for (void* o : outs)
-    if (o && (!is_device_pointer(o) || on_other_device(o, map->device)))
+  for (void* o : outs) {
+    const Where w = where_is(o, map->device);
+    if (o && (!w.device || w.other))
       return fail(OHM_ERR_INVALID, "export: outputs must be device memory of the map's device");
+  }
   if (path_sum && !(map->p.layers & OHM_LAYER_DECAY)) return fail(OHM_ERR_UNSUPPORTED, "export: no decay layer");
   if (mean && !(map->p.layers & OHM_LAYER_MEAN)) return fail(OHM_ERR_UNSUPPORTED, "export: no mean layer");
   if (occupancy && !(map->p.layers & OHM_LAYER_OCCUPANCY)) return fail(OHM_ERR_UNSUPPORTED, "export: no occupancy layer");

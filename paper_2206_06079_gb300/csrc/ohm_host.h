@@ -36,7 +36,8 @@ struct ohm_map {
   cudaEvent_t hin_free[2];    // kernels of the slot's last call done
   int hin_next;
   // pinned host mirrors for status / counters
-  int32_t* h_status;
+  int32_t* h_status;        // [0] copies of the device word, [1] DeviceMap::host_status
+  bool status_copied;       // h_status[1] holds (once the stream has passed) what the device word holds
   ohm::CallCounters* h_calls;
   int32_t* h_count;
   long long launches;       // kernels launched by this map

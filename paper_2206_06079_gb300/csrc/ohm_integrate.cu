@@ -350,6 +350,7 @@ cudaError_t launch_integrate(ohm_map* map, const CallArgs& args, cudaStream_t st
   const int ray_grid = (int)(per_ray_blocks < grid ? per_ray_blocks : grid);
   const unsigned prb = (unsigned)per_ray_blocks;
   map->last_rays = n;
+  map->status_copied = true;
   if (occ_like) {
     OHM_LAUNCH(OHM_STAGE_PREPARE, launch_chained(k_prepare_occ, prb, stream, m, args));
     if (ndt) OHM_LAUNCH(OHM_STAGE_NDT_ALLOC, launch_chained(k_ndt_alloc, kNdtPendingGrid, stream, m));

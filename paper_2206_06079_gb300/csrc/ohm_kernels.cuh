@@ -308,10 +308,13 @@ __device__ __forceinline__ void finish_call(const DeviceMap& m) {
   c->restores = 0;
   c->ndt_pending = 0;
   c->mean_touched = 0;
-  if (!latched(m)) {
+  const int32_t status = *(volatile int32_t*)m.status;
+  if (status == 0) {
     c->seq += 1;
     snapshot_pool(m);
   }
+  // read by ohm_map_sync without a copy of its own
+  *(volatile int32_t*)m.host_status = status;
 }
 
 // Fixed-point origin of the current call's rays where they share one: the
