@@ -471,13 +471,12 @@ ohm_status ohm_batch_stats(ohm_batch* batch, int64_t* kernel_launches, int64_t* 
  * has one) gets hits += 1.  Voxels outside the grid are not counted.
  *
  * It allocates nothing: its working memory is one statically sized device
- * array inside the library (about 3 MB), which every GPU that loads the library
+ * array inside the library (2 MB), which every GPU that loads the library
  * holds until the process exits.  The first call on a device looks up that
  * array's device address (cudaGetSymbolAddress); make that first call before
  * any stream capture.  Every call uses the calling thread's current device and
  * shares the array: calls whose work may overlap on the GPU (unordered streams)
- * race on it and must not be issued.  Each call clears the part that must start
- * at zero.  All pointers must be device memory of the current device; hits and
+ * race on it and must not be issued.  All pointers must be device memory of the current device; hits and
  * misses must each hold dims[0] * dims[1] * dims[2] uint32 elements and flags
  * (if not NULL) n bytes -- the library cannot check the sizes of caller
  * buffers, and a short one is written or read out of bounds.
@@ -492,7 +491,7 @@ typedef struct {
   double voxel_size;       /* voxel edge in metres */
   double map_origin[3];    /* world position of the lower corner of voxel (0,0,0) */
   int32_t frac_bits;       /* fixed-point fraction bits per voxel, 8..20 */
-  int32_t segment_steps;   /* ray segment length in dominant-axis steps; 0 = 64 */
+  int32_t segment_steps;   /* ray segment length in dominant-axis steps (enters the size limit); 0 = 64 */
   double max_range;        /* truncation length in metres */
   int64_t corner[3];       /* voxel index of grid cell (0,0,0) */
   int64_t dims[3];         /* grid size in voxels; cell (x,y,z) is element x + dims[0] * (y + dims[1] * z) */
