@@ -89,7 +89,7 @@ __device__ __forceinline__ long long point_offset(const DeviceMap& m, const floa
   long long q[3];
   bool ok = true;
 #pragma unroll
-  for (int k = 0; k < 3; ++k) ok = ok && isfinite(p[k]) && quantise(p[k], m.origin[k], m.scale, &q[k]);
+  for (int k = 0; k < 3; ++k) ok = quantise_coord(m, p[k], k, &q[k]) && ok;
   ok = ok && in_extent(q, m.frac_bits);
   if (!ok) return -1;
   const int F = m.frac_bits;
@@ -259,7 +259,7 @@ __device__ __forceinline__ float* ndt_grad_of(const DeviceMap& m, const float* p
   long long q[3];
   bool ok = true;
 #pragma unroll
-  for (int k = 0; k < 3; ++k) ok = ok && isfinite(p[k]) && quantise(p[k], m.origin[k], m.scale, &q[k]);
+  for (int k = 0; k < 3; ++k) ok = quantise_coord(m, p[k], k, &q[k]) && ok;
   ok = ok && in_extent(q, m.frac_bits);
   if (!ok) return nullptr;
   const int F = m.frac_bits;

@@ -316,10 +316,23 @@ ohm_status ohm_map_create(const ohm_map_params* params, ohm_map** out) {
     // |b - a|^2 <= (rmax_q - 1)^2 gives a double length below rmax_q (its
     // relative error is a few 2^-53); checked against the double bound
     const double r_in = d.rmax_q - 1.0;
-    d.rmax_in2 = r_in > 0.0 ? (unsigned long long)std::floor(r_in * r_in) : 0ULL;
+    d.rmax_safe2 = r_in > 0.0 ? (unsigned long long)std::floor(r_in * r_in) : 0ULL;
+    // the largest integer up to 2^53 whose double square root is at most
+    // rmax_q (the square root is monotone: a binary search)
+    unsigned long long lo = 0, hi = 1ULL << 53;
+    while (lo < hi) {
+      const unsigned long long mid = lo + (hi - lo + 1) / 2;
+      if (std::sqrt((double)mid) <= d.rmax_q)
+        lo = mid;
+      else
+        hi = mid - 1;
+    }
+    d.rmax_in2 = lo;
   }
   d.rmin_q = p.min_range * scale;
   d.tau_q = p.tsdf_trunc * scale;
+  for (int k = 0; k < 3; ++k) d.origin_ff[k] = ohm::ff_of_double(p.map_origin[k]);
+  d.scale_ff = ohm::ff_of_double(scale);
   d.band.tau = ohm::ff_of_double(d.tau_q);
   d.band.rmin = ohm::ff_of_double(d.rmin_q);
   d.band.rmax = ohm::ff_of_double(d.rmax_q);

@@ -191,9 +191,11 @@ struct DeviceMap {
   double scale;                  // 2^F / voxel_size
   double rmax_q, rmin_q, tau_q;  // ranges in fixed-point units
   BandConsts band;               // tau_q, rmin_q, rmax_q as float-float
-  // a ray with |b - a|^2 <= rmax_in2 (fixed-point units^2) is certainly
-  // within max_range
-  unsigned long long rmax_in2;
+  FF origin_ff[3], scale_ff;     // origin and scale as float-float
+  // a ray with |b - a|^2 <= rmax_safe2 (fixed-point units^2) is certainly
+  // within max_range; rmax_in2: the largest |b - a|^2 up to 2^53 whose double
+  // square root does not exceed rmax_q
+  unsigned long long rmax_safe2, rmax_in2;
   double voxel_size;
   int32_t frac_bits;
   uint32_t layers;
@@ -1335,6 +1337,62 @@ __host__ __device__ __forceinline__ bool ff_to_float(FF q, float e, float* out) 
   *out = q.hi;
   return true;
 }
+// A 32-bit integer as float-float, exactly.
+__host__ __device__ __forceinline__ FF ff_of_int(int32_t v) {
+  const float hi = (float)v;
+  return {hi, (float)(v - (int32_t)hi)};
+}
+
+// rint(s) of a float-float s with |s| < 2^27, as ff_rint (below) does for
+// |x| < 2^25: the low part may itself be a few units.
+__host__ __device__ __forceinline__ bool ff_rint_wide(FF s, float e, int32_t* out) {
+  const float n = rintf(s.hi);
+  const float t = fadd_rn(fsub_rn(s.hi, n), s.lo);  // |t| < 5: one rounding below 2.4e-7
+  const float n2 = rintf(t);
+  if (!(fabsf(fsub_rn(t, n2)) < 0.5f - (e + 1e-6f))) return false;
+  *out = (int32_t)n + (int32_t)n2;
+  return true;
+}
+
+// quantise() settled in float-float: rint(fl(fl(x - origin) scale)) when no
+// half-integer lies within E = 2^-44 (|x| + |origin|) scale of the float-float
+// value; else false, and the caller evaluates in double.  Against the exact
+// (x - origin) scale the double evaluation is off by less than 2^-52 of it; the
+// float-float one by u^2 |origin| (its 48 bits) and 3 u^2 (|x| + |origin|) in
+// the difference, u^2 in scale and 5 u^2 in the product, together below 10 u^2
+// (|x| + |origin|) scale = 0.63 E.  |s| < 2^27 is tested first (false for NaN).
+// Four double instructions per coordinate cost a warp 64 cycles of a
+// scheduler each; this is 25 float ones.
+__host__ __device__ __forceinline__ bool quantise_ff(float x, FF origin, FF scale, long long* q) {
+  FF d = two_sum(x, -origin.hi);
+  d = fast_two_sum(d.hi, fsub_rn(d.lo, origin.lo));
+  const FF s = ff_mul(d, scale);
+  if (!(fabsf(s.hi) < 134217728.0f)) return false;
+  const float e = 5.684342e-14f * (fabsf(x) + fabsf(origin.hi)) * scale.hi;
+  int32_t v;
+  if (!ff_rint_wide(s, e, &v)) return false;
+  *q = v;
+  return true;
+}
+
+// Truncation of a ray longer than max_range, qe_k = qo_k + rint(fl(d_k
+// fl(rmax / len))), len = fl(sqrt(l2)) with l2 = |d|^2 < 2^53 exact, settled in
+// float-float: len to 5 u^2 (l2's 48 bits and ff_sqrt), 1 / len to 11 u^2,
+// rmax / len to 17 u^2, the products to 23 u^2 of |d_k|; the double evaluation's
+// three roundings add 2^-51.  Each end point is taken when no half-integer
+// lies within 2^-40 |d_k| (256 u^2) of it; else false (nothing is written).
+__host__ __device__ __forceinline__ bool truncate_ff(const int32_t d[3], unsigned long long l2, FF rmax, int32_t out[3]) {
+  const float h = (float)l2;
+  const FF L = fast_two_sum(h, (float)(long long)(l2 - (unsigned long long)h));
+  const FF ratio = ff_mul(rmax, ff_rcp(ff_sqrt(L)));
+OHM_UNROLL
+  for (int k = 0; k < 3; ++k) {
+    const FF p = ff_mul(ratio, ff_of_int(d[k]));
+    if (!(fabsf(p.hi) < 134217728.0f) || !ff_rint_wide(p, 9.094947e-13f * fabsf((float)d[k]), &out[k])) return false;
+  }
+  return true;
+}
+
 // ---------------------------------------------------------------------------
 // The TSDF band of tsdf_band (with its range test len > rmin, len <= rmax on
 // the double length of ray_length) settled in float-float arithmetic, for

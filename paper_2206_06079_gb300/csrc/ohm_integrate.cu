@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(kBlock) k_query(DeviceMap m, const float* pts,
   long long q[3];
   bool ok = true;
 #pragma unroll
-  for (int k = 0; k < 3; ++k) ok = ok && isfinite(pts[3 * i + k]) && quantise(pts[3 * i + k], m.origin[k], m.scale, &q[k]);
+  for (int k = 0; k < 3; ++k) ok = quantise_coord(m, pts[3 * i + k], k, &q[k]) && ok;
   ok = ok && in_extent(q, F);
   int32_t slot = -1;
   uint32_t mo = 0;

@@ -74,6 +74,13 @@ __device__ __forceinline__ float logodds_value(float s, float l_min) { return s 
 // below l_min reads as l_min.
 __device__ __forceinline__ float logodds_read(float s, float l_min) { return s < l_min ? l_min : s; }
 
+// One coordinate of a point: quantise(), in float-float where that settles it.
+// Returns false for a non-finite coordinate too.
+__device__ __forceinline__ bool quantise_coord(const DeviceMap& m, float x, int k, long long* q) {
+  if (quantise_ff(x, m.origin_ff[k], m.scale_ff, q)) return true;
+  return isfinite(x) && quantise(x, m.origin[k], m.scale, q);
+}
+
 // Quantise a ray, returns false when it is skipped (non-finite coordinate or
 // a point beyond the fixed-point range).
 __device__ __forceinline__ bool quantise_ray(const DeviceMap& m, const float o[3], const float e[3], long long qo[3],
@@ -81,9 +88,8 @@ __device__ __forceinline__ bool quantise_ray(const DeviceMap& m, const float o[3
   bool ok = true;
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    ok = ok && isfinite(o[k]) && isfinite(e[k]);
-    ok = ok && quantise(o[k], m.origin[k], m.scale, &qo[k]);
-    ok = ok && quantise(e[k], m.origin[k], m.scale, &qe[k]);
+    ok = quantise_coord(m, o[k], k, &qo[k]) && ok;
+    ok = quantise_coord(m, e[k], k, &qe[k]) && ok;
   }
   return ok;
 }
@@ -330,7 +336,8 @@ __device__ __forceinline__ CallOrigin call_origin(const DeviceMap& m, const Call
   const int lane = threadIdx.x & 31, k = lane < 3 ? lane : 2;
   const float o = a.origins[k];
   long long q = 0;
-  const bool ok = isfinite(o) && quantise(o, k == 0 ? m.origin[0] : (k == 1 ? m.origin[1] : m.origin[2]), m.scale, &q);
+  bool ok = quantise_ff(o, k == 0 ? m.origin_ff[0] : (k == 1 ? m.origin_ff[1] : m.origin_ff[2]), m.scale_ff, &q);
+  if (!ok) ok = isfinite(o) && quantise(o, k == 0 ? m.origin[0] : (k == 1 ? m.origin[1] : m.origin[2]), m.scale, &q);
 #pragma unroll
   for (int i = 0; i < 3; ++i) r.q[i] = __shfl_sync(full, q, i);
   r.ok = __all_sync(full, ok);
@@ -347,7 +354,7 @@ __device__ __forceinline__ bool quantise_call_ray(const DeviceMap& m, const Call
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     qo[k] = origin.q[k];
-    ok = ok && isfinite(e[k]) && quantise(e[k], m.origin[k], m.scale, &qe[k]);
+    ok = quantise_coord(m, e[k], k, &qe[k]) && ok;
   }
   return ok;
 }
@@ -402,19 +409,36 @@ __device__ __forceinline__ void prepare_occ_ray(const DeviceMap& m, const CallAr
     bool ok = quantise_call_ray(m, args, origin, o, e, qo, qe);
     bool sample = (flag & kFlagNoReturn) == 0;
     if (ok) {
-      // Truncation test len > rmax_q with len the double length: settled by
-      // the exact integer |b - a|^2 unless it lies in a band around rmax_q^2
-      // (or an axis difference is too large for it), where the double
-      // evaluation decides.
-      bool in_range = false;
+      // Truncation test len > rmax_q with len the double length.  Up to 2^53
+      // the squared length is exact in double as in integers, so the test is
+      // one on integers; the truncated end point is formed in float-float
+      // where that settles it.  A missing return lies within rounding of the
+      // range limit, so half of them come here, and a warp that holds one ran
+      // a double square root and division for all its lanes.
+      bool done = false;
       const long long dx = qe[0] - qo[0], dy = qe[1] - qo[1], dz = qe[2] - qo[2];
       const long long lim = 1LL << 30;
       if (dx > -lim && dx < lim && dy > -lim && dy < lim && dz > -lim && dz < lim) {
         const unsigned long long l2 = (unsigned long long)(dx * dx) + (unsigned long long)(dy * dy) +
                                       (unsigned long long)(dz * dz);
-        in_range = l2 <= m.rmax_in2;
+        if (l2 <= m.rmax_safe2) {
+          done = true;
+        } else if (l2 < (1ULL << 53)) {  // every difference below 2^27
+          if (l2 <= m.rmax_in2) {
+            done = true;
+          } else {
+            const int32_t d[3] = {(int32_t)dx, (int32_t)dy, (int32_t)dz};
+            int32_t cut[3];
+            if (truncate_ff(d, l2, m.band.rmax, cut)) {
+#pragma unroll
+              for (int k = 0; k < 3; ++k) qe[k] = qo[k] + cut[k];
+              sample = false;
+              done = true;
+            }
+          }
+        }
       }
-      if (!in_range) {
+      if (!done) {
         double d[3];
         const double len = ray_length(qo, qe, d);
         if (len > m.rmax_q) {
