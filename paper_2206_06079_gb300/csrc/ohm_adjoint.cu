@@ -41,21 +41,48 @@ struct DepthFrame {
   double R[9];
   double t[3];
   double z_min, z_max;
+  float z_lo, z_hi;   // the largest floats up to z_min and z_max: a float z has z > z_min iff z > z_lo
+  FF Rf[9], tf[3], zf_max;  // R, t and z_max as float-float
   const double* pxy;  // (u - cx) / fx for u < width, then (v - cy) / fy for v < height
+  const float2* pxyf; // the same as float-float (hi, lo)
 };
+
+// Pixel of the i-th thread of a frame, so that a warp holds an 8 x 4 tile: its
+// rays stay within a voxel or two of one another, where 32 pixels of a row
+// spread over several (the TSDF walk then has more voxels per step to update).
+// Rows in bands of 4 (the last may be lower), columns in tiles of 8, the
+// columns left over behind them.
+__device__ __forceinline__ long long tile_pixel(long long p, int width, int height) {
+  if ((long long)width * height >= (1LL << 31)) return p;  // row by row
+  const int i = (int)p;
+  const int band = i / (4 * width), rows = height - 4 * band < 4 ? height - 4 * band : 4;
+  const int t = i - band * 4 * width, tiles = width / 8, in_tiles = tiles * 8 * rows;
+  int row, col;
+  if (t < in_tiles) {
+    const int tile = t / (8 * rows), r = t - tile * 8 * rows;
+    row = r / 8;
+    col = tile * 8 + (r & 7);
+  } else {
+    const int rest = width - 8 * tiles, r = t - in_tiles;
+    row = r / rest;
+    col = 8 * tiles + r - row * rest;
+  }
+  return (long long)(4 * band + row) * width + col;
+}
 
 // Back-projection of one pixel, one rounding per double operation:
 // x = ((u - cx) / fx) z, y = ((v - cy) / fy) z, e_k = ((R_k0 x + R_k1 y) + R_k2 z) + t_k,
 // rounded to float.  A depth outside (z_min, z_max] gives a NO_RETURN ray at z_max.
 // The quotients depend on the column or the row only: they come from the
 // frame's table, formed on the host by the same double operations.
-__device__ __forceinline__ bool depth_ray(const DepthFrame& f, long long pix, float e[3], double pt[3]) {
-  const int u = (int)(pix % f.width), v = (int)(pix / f.width);
-  const double z = (double)f.depth[pix];
-  const bool valid = z > f.z_min && z <= f.z_max;
-  const double zz = valid ? z : f.z_max;
-  const double px = f.pxy[u];
-  const double py = f.pxy[f.width + v];
+//
+// Evaluated in float-float first: with S_k = |R_k0 x| + |R_k1 y| + |R_k2 z| +
+// |t_k|, x and y are good to 6 u^2 (their quotient's 48 bits and one product),
+// the products by R to 13 u^2, and the three additions and t add 10 u^2 S_k; the
+// double evaluation is within 2^-50 S_k. The float is taken when no midpoint
+// between floats lies within 2^-41 S_k = 128 u^2 S_k; else the pixel is
+// evaluated in double (20 double instructions, 64 scheduler cycles each).
+__device__ __noinline__ void depth_ray_double(const DepthFrame& f, double px, double py, double zz, float e[3]) {
   const double x = __dmul_rn(px, zz), y = __dmul_rn(py, zz);
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
@@ -65,9 +92,26 @@ __device__ __forceinline__ bool depth_ray(const DepthFrame& f, long long pix, fl
     a = __dadd_rn(a, f.t[k]);
     e[k] = __double2float_rn(a);
   }
-  pt[0] = px;
-  pt[1] = py;
-  pt[2] = 1.0;
+}
+__device__ __forceinline__ bool depth_ray(const DepthFrame& f, long long pix, float e[3], float* px, float* py) {
+  const int v = pix < (1LL << 31) ? (int)pix / f.width : (int)(pix / f.width);
+  const int u = (int)(pix - (long long)v * f.width);
+  const float z = f.depth[pix];
+  const bool valid = z > f.z_lo && z <= f.z_hi;
+  const float2 qx = f.pxyf[u], qy = f.pxyf[f.width + v];
+  const FF X = {qx.x, qx.y}, Y = {qy.x, qy.y}, Z = valid ? FF{z, 0.0f} : f.zf_max;
+  const FF x = ff_mul(X, Z), y = ff_mul(Y, Z);
+  bool settled = true;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const FF a = ff_mul(f.Rf[3 * k], x), b = ff_mul(f.Rf[3 * k + 1], y), c = ff_mul(f.Rf[3 * k + 2], Z);
+    const FF s = ff_add(ff_add(ff_add(a, b), c), f.tf[k]);
+    const float S = fabsf(a.hi) + fabsf(b.hi) + fabsf(c.hi) + fabsf(f.tf[k].hi);
+    settled = ff_to_float(s, 4.547474e-13f * S, &e[k]) && S < 1e18f && settled;
+  }
+  if (!settled) depth_ray_double(f, f.pxy[u], f.pxy[f.width + v], valid ? (double)z : f.z_max, e);
+  *px = qx.x;
+  *py = qy.x;
   return valid;
 }
 
@@ -75,9 +119,8 @@ __global__ void __launch_bounds__(kBlock) k_depth_rays(DepthFrame f, float* orig
   const long long n = (long long)f.width * f.height;
   if (blockIdx.x == 0 && threadIdx.x < 3) origins[threadIdx.x] = __double2float_rn(f.t[threadIdx.x]);
   for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x) {
-    float e[3];
-    double pt[3];
-    const bool valid = depth_ray(f, p, e, pt);
+    float e[3], px, py;
+    const bool valid = depth_ray(f, tile_pixel(p, f.width, f.height), e, &px, &py);
     endpoints[3 * p + 0] = e[0];
     endpoints[3 * p + 1] = e[1];
     endpoints[3 * p + 2] = e[2];
@@ -117,99 +160,93 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-__global__ void __launch_bounds__(kBlock) k_tsdf_backward(DeviceMap m, DepthFrame f, float* grad_depth,
+// Compiled for 2 blocks per SM (128 registers; 184 unbounded, which fits one;
+// 3 and 4 blocks: no difference).  640 x 480 frame with 20,000 queries: 121 us with
+// the double back-projection and the 64-bit walker, row by row; 100 us now.
+__global__ void __launch_bounds__(kBlock, 2) k_tsdf_backward(DeviceMap m, DepthFrame f, float* grad_depth,
                                                           double* grad_twist) {
   __shared__ double red[kBlock / 32][6];
+  __shared__ uint32_t tabs[8 * kBlock];
+  uint32_t* const tab = tabs + threadIdx.x;
   const long long n = (long long)f.width * f.height;
   const int F = m.frac_bits;
-  const long long U = 1LL << F;
-  const long long half = U >> 1;
-  const float to_m = (float)(m.voxel_size / (double)U);
+  const float to_m = (float)(m.voxel_size / (double)(1LL << F));
+  const float O[3] = {(float)f.t[0], (float)f.t[1], (float)f.t[2]};
   double acc[6] = {0, 0, 0, 0, 0, 0};
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  const long long n_round = (n + stride - 1) / stride * stride;  // whole blocks iterate together
-  for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < n_round; p += stride) {
+  for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x) {
+    const long long pix = tile_pixel(p, f.width, f.height);
     float gz = 0.f;
-    if (p < n) {
-      float e[3], o[3];
-      double pt[3];
-      bool ok = depth_ray(f, p, e, pt);
+    float e[3], px, py;
+    bool ok = depth_ray(f, pix, e, &px, &py);
+    long long qo[3], qe[3], a[3], b[3];
+    float u[3], lenf = 0.f;
+    // the band of the forward pass, recomputed the same way
+    ok = ok && quantise_ray(m, O, e, qo, qe) && tsdf_ray_band(m, qo, qe, a, b, u, &lenf);
+    if (ok) {
+      const float dm = lenf * to_m;  // ray length in metres (chain rule only)
+      TsdfRec t;
+      tsdf_record(a, b, qe, F, &t);
+      const int M = (t.r.flags >> kRayAxisShift) & 3;
+      const int32_t nmaj = M == 0 ? t.r.n[0] : (M == 1 ? t.r.n[1] : t.r.n[2]);
+      float A = 0.f, B[3] = {0.f, 0.f, 0.f};
+      for (int32_t K = 0; K <= nmaj; K += kPieceSlots) {
+        const int32_t Ke = K + kPieceSlots < nmaj + 1 ? K + kPieceSlots : nmaj + 1;
+        PieceStart ps;
+        LWalker w;
+        uint32_t mo;
+        piece_start(t.r, F, K, Ke, Ke == nmaj + 1, &ps, &w);
+        if (!piece_regions(m, ps, w, t.r.flags, tab, &mo)) break;  // not integrated: nothing to differentiate
+        int32_t rel[3];
 #pragma unroll
-      for (int k = 0; k < 3; ++k) o[k] = __double2float_rn(f.t[k]);
-      long long qo[3], qe[3];
-      ok = ok && quantise_ray(m, o, e, qo, qe);
-      // the band of the forward pass, recomputed the same way
-      long long a[3], b[3];
-      float u[3], lenf = 0.f;
-      if (ok) {
-        bool in_range = false;
-        if (!tsdf_band_ff(qo, qe, m.band, &in_range, a, b, u, &lenf)) {
-          double d[3];
-          const double len = ray_length(qo, qe, d);
-          in_range = len > m.rmin_q && len <= m.rmax_q;
-          if (in_range && in_extent(qo, F) && in_extent(qe, F)) tsdf_band(qo, d, len, m.tau_q, a, b, u);
-          lenf = (float)len;
-        }
-        ok = in_range && in_extent(qo, F) && in_extent(qe, F);
-      }
-      if (ok) {
-        const float dm = lenf * to_m;  // ray length in metres (chain rule only)
-        Walker w;
-        walker_init(w, a, b, F, 0, 0);
-        int32_t slot = region_slot_of(m, w.vx, w.vy, w.vz);
-        uint32_t mo = local_morton(w.vx, w.vy, w.vz);
-        float A = 0.f, B[3] = {0.f, 0.f, 0.f};
-        while (slot >= 0) {
-          const long long off = voxel_offset(slot, mo);
-          const float G = m.grad[off];
-          if (G != 0.f) {
-            const float ex = (float)(qe[0] - ((long long)w.vx * U + half));
-            const float ey = (float)(qe[1] - ((long long)w.vy * U + half));
-            const float ez = (float)(qe[2] - ((long long)w.vz * U + half));
-            const float s = (ex * u[0] + ey * u[1] + ez * u[2]) * to_m;  // as in the forward pass
-            if (s > -m.tau_m && s < m.tau_m) {
-              const float wv = G / m.tsdf[off].y;
-              const float r[3] = {ex * to_m, ey * to_m, ez * to_m};
-              A += wv;
+        for (int k = 0; k < 3; ++k) rel[k] = t.e[k] - ((ps.v[k] - t.r.v0[k]) << F);
+        for (int32_t left = ps.visits; left > 0;) {
+          uint32_t at[kFastBatch], off[kFastBatch], valid;
+          float G[kFastBatch];
+          piece_fill(m, &t.r, K, tab, w, mo, left, at, off, valid);
 #pragma unroll
-              for (int k = 0; k < 3; ++k) B[k] += wv * (r[k] - s * u[k]);
+          for (int j = 0; j < kFastBatch; ++j) G[j] = ((valid >> j) & 1u) ? m.grad[off[j]] : 0.f;
+#pragma unroll
+          for (int j = 0; j < kFastBatch; ++j) {
+            if (G[j] != 0.f) {
+              const float ex = (float)rel[0], ey = (float)rel[1], ez = (float)rel[2];
+              const float s = (ex * u[0] + ey * u[1] + ez * u[2]) * to_m;  // as in the forward pass
+              if (s > -m.tau_m && s < m.tau_m) {
+                const float wv = G[j] / m.tsdf[off[j]].y;
+                const float r[3] = {ex * to_m, ey * to_m, ez * to_m};
+                A += wv;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) B[k] += wv * (r[k] - s * u[k]);
+              }
             }
+            const uint32_t moved = at[j] ^ (j + 1 < kFastBatch ? at[j + 1] : mo);
+            const int k = (moved & 0x9249u) ? 0 : ((moved & 0x12492u) ? 1 : 2);
+            const int32_t d = ((t.r.flags >> (kRaySignShift + k)) & 1) ? 1 << F : -(1 << F);
+            rel[0] += k == 0 ? d : 0;
+            rel[1] += k == 1 ? d : 0;
+            rel[2] += k == 2 ? d : 0;
           }
-          if (w.total == 0) break;
-          const int axis = walker_choose(w);
-          int32_t c, sg;
-          walker_step(w, axis, &c, &sg);
-          mo = morton_step(mo, morton_mask(axis), sg);
-          if ((c & ((1 << kRegionShift) - 1)) == (sg > 0 ? 0 : (1 << kRegionShift) - 1))
-            slot = region_slot_of(m, w.vx, w.vy, w.vz);
         }
-        // The chain rule from here on is plain float arithmetic (its inputs
-        // are floats; the gradients are checked to 1e-3 relative), summed
-        // over pixels in double.  The band above is recomputed exactly as
-        // the forward pass forms it (the same float-float settlement, else
-        // the same double evaluation), since it decides the voxel set.
-        const float rdm = 1.0f / dm;
-        float ge[3], go[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          go[k] = -B[k] * rdm;
-          ge[k] = A * u[k] - go[k];
-        }
-        const float ptf[3] = {(float)pt[0], (float)pt[1], (float)pt[2]};
-        float dz = 0.f;
-#pragma unroll
-        for (int k = 0; k < 3; ++k)
-          dz += ge[k] * ((float)f.R[3 * k] * ptf[0] + (float)f.R[3 * k + 1] * ptf[1] + (float)f.R[3 * k + 2] * ptf[2]);
-        gz = dz;
-        const float O[3] = {(float)f.t[0], (float)f.t[1], (float)f.t[2]};
-#pragma unroll
-        for (int k = 0; k < 3; ++k) acc[k] += (double)(ge[k] + go[k]);
-        acc[3] += (double)(e[1] * ge[2] - e[2] * ge[1] + O[1] * go[2] - O[2] * go[1]);
-        acc[4] += (double)(e[2] * ge[0] - e[0] * ge[2] + O[2] * go[0] - O[0] * go[2]);
-        acc[5] += (double)(e[0] * ge[1] - e[1] * ge[0] + O[0] * go[1] - O[1] * go[0]);
       }
-      grad_depth[p] = gz;
+      // The chain rule from here on is plain float arithmetic (its inputs
+      // are floats; the gradients are checked to 1e-3 relative), summed
+      // over pixels in double.  The band above is recomputed exactly as
+      // the forward pass forms it, since it decides the voxel set.
+      const float rdm = 1.0f / dm;
+      float ge[3], go[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        go[k] = -B[k] * rdm;
+        ge[k] = A * u[k] - go[k];
+      }
+#pragma unroll
+      for (int k = 0; k < 3; ++k) gz += ge[k] * (f.Rf[3 * k].hi * px + f.Rf[3 * k + 1].hi * py + f.Rf[3 * k + 2].hi);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) acc[k] += (double)(ge[k] + go[k]);
+      acc[3] += (double)(e[1] * ge[2] - e[2] * ge[1] + O[1] * go[2] - O[2] * go[1]);
+      acc[4] += (double)(e[2] * ge[0] - e[0] * ge[2] + O[2] * go[0] - O[0] * go[2]);
+      acc[5] += (double)(e[0] * ge[1] - e[1] * ge[0] + O[0] * go[1] - O[1] * go[0]);
     }
+    grad_depth[pix] = gz;
   }
   // block reduction of the twist gradient, one double atomic per component
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -380,7 +417,17 @@ bool frame_from(const float* depth, int32_t width, int32_t height, const double*
   }
   f->z_min = z_min;
   f->z_max = z_max;
+  auto below = [](double z) {  // the largest float not above z
+    float r = (float)z;
+    return (double)r > z ? std::nextafter(r, -INFINITY) : r;
+  };
+  f->z_lo = below(z_min);
+  f->z_hi = below(z_max);
+  for (int k = 0; k < 9; ++k) f->Rf[k] = ff_of_double(f->R[k]);
+  for (int k = 0; k < 3; ++k) f->tf[k] = ff_of_double(f->t[k]);
+  f->zf_max = ff_of_double(z_max);
   f->pxy = nullptr;
+  f->pxyf = nullptr;
   return f->fx != 0.0 && f->fy != 0.0;
 }
 
@@ -388,33 +435,40 @@ bool frame_from(const float* depth, int32_t width, int32_t height, const double*
 // last image size and intrinsics (rebuilt when they change).
 cudaError_t frame_tables(ohm_map* map, DepthFrame* f, cudaStream_t s) {
   const double key[6] = {(double)f->width, (double)f->height, f->fx, f->fy, f->cx, f->cy};
-  const long long n = (long long)f->width + f->height;
+  const long long n = (long long)f->width + f->height;  // doubles, then as many float pairs
   if (map->pxy && std::memcmp(key, map->pxy_key, sizeof(key)) == 0) {
     f->pxy = map->pxy;
+    f->pxyf = reinterpret_cast<const float2*>(map->pxy + n);
     return cudaSuccess;
   }
   // earlier work of the map may still read the old table
   cudaError_t e = map->work_done ? cudaStreamWaitEvent(s, map->work_done, 0) : cudaSuccess;
-  if (e == cudaSuccess && n > map->pxy_cap) {
+  if (e == cudaSuccess && 2 * n > map->pxy_cap) {
     if (map->pxy) {
       e = cudaStreamSynchronize(s);
       if (e == cudaSuccess) e = cudaFree(map->pxy);
       map->pxy = nullptr;
       map->pxy_cap = 0;
     }
-    const long long cap = n > 4096 ? n : 4096;
+    const long long cap = 2 * n > 8192 ? 2 * n : 8192;
     if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&map->pxy), sizeof(double) * cap);
     if (e != cudaSuccess) return e;
     map->pxy_cap = cap;
   }
   if (e != cudaSuccess) return e;
-  std::vector<double> t((size_t)n);
+  std::vector<double> t((size_t)(2 * n));
   for (int u = 0; u < f->width; ++u) t[u] = ((double)u - f->cx) / f->fx;
   for (int v = 0; v < f->height; ++v) t[f->width + v] = ((double)v - f->cy) / f->fy;
-  e = cudaMemcpyAsync(map->pxy, t.data(), sizeof(double) * n, cudaMemcpyHostToDevice, s);
+  for (long long k = 0; k < n; ++k) {
+    const FF q = ff_of_double(t[(size_t)k]);
+    const float pair[2] = {q.hi, q.lo};
+    std::memcpy(&t[(size_t)(n + k)], pair, sizeof(pair));
+  }
+  e = cudaMemcpyAsync(map->pxy, t.data(), sizeof(double) * 2 * n, cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return e;
   std::memcpy(map->pxy_key, key, sizeof(key));
   f->pxy = map->pxy;
+  f->pxyf = reinterpret_cast<const float2*>(map->pxy + n);
   return cudaSuccess;
 }
 

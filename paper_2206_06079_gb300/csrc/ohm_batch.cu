@@ -213,16 +213,19 @@ __global__ void __launch_bounds__(kBlock) k_batch_mean_apply(const BatchDesc* de
   }
 }
 
-__global__ void __launch_bounds__(kBlock) k_batch_tsdf_walk(const BatchDesc* desc, const BatchStep* step) {
+__global__ void __launch_bounds__(kBlock, 4) k_batch_tsdf_walk(const BatchDesc* desc, const BatchStep* step) {
   chain_enter();
   __shared__ BatchShared sh;
+  __shared__ uint32_t tab[8 * kBlock];
+  __shared__ uint32_t acc[2 * kBlock];
+  acc[threadIdx.x] = acc[kBlock + threadIdx.x] = 0;  // batch_stage synchronises the block
   batch_stage(sh, desc, step, kRaysPadded);
   const long long total = sh.pref[sh.n_maps];  // a multiple of 32: whole warps iterate together
   OHM_BATCH_STRIDE(g, total) {
     const int mi = batch_find(sh, g);
     const DeviceMap& m = sh.maps[mi];
     const long long i = g - sh.pref[mi];
-    if (m.layers & kLayerTsdf) tsdf_walk_ray(m, i, i < step->n[mi] && !latched(m));
+    if (m.layers & kLayerTsdf) tsdf_walk_ray(m, i, i < step->n[mi] && !latched(m), tab + threadIdx.x, acc + 2 * (threadIdx.x & ~31u));
   }
 }
 

@@ -96,13 +96,12 @@ struct __align__(16) EndpointRec {
 };
 
 // Ray record written by the TSDF prepare kernel: the walk covers the band
-// [max(0, d - tau), d + tau] of the ray from the sensor to the sample e.
+// [max(0, d - tau), d + tau] of the ray from the sensor to the sample.
 struct __align__(16) TsdfRec {
-  long long a[3];   // band start, fixed point
-  long long b[3];   // band end, fixed point
-  long long e[3];   // sample, fixed point
+  RayRec r;         // the band's walk constants (kRayValid when the ray updates the TSDF; inv only
+                    // where the band is longer than one piece of the local walk)
+  int32_t e[3];     // sample minus the centre of the band's first voxel, fixed point
   float u[3];       // unit direction sensor -> sample
-  int32_t flags;    // kRayValid when the ray updates the TSDF
 };
 
 // Per-call counters in device memory.
@@ -1302,7 +1301,7 @@ __host__ __device__ __forceinline__ bool ff_rint(FF x, float e, long long* out) 
   const float n = rintf(x.hi);                         // an integer within 1/2 of x.hi
   const float f = fadd_rn(fsub_rn(x.hi, n), x.lo);     // x - n, one rounding (|f| <= 1.5)
   const float m = e + 1e-6f;                           // covers the rounding of f
-  long long k = (long long)n;
+  int32_t k = (int32_t)n;
   if (fabsf(f) < 0.5f - m) {
   } else if (f > 0.5f + m && f < 1.5f - m) {
     k += 1;
@@ -1423,7 +1422,7 @@ OHM_UNROLL
   for (int k = 0; k < 3; ++k) {
     const long long dk = qe[k] - qo[k];
     if (dk <= -(1LL << 24) || dk >= (1LL << 24)) return false;
-    d[k] = (float)dk;
+    d[k] = (float)(int32_t)dk;
   }
   const FF S = ff_add(ff_add(two_prod(d[0], d[0]), two_prod(d[1], d[1])), two_prod(d[2], d[2]));
   if (!(S.hi > 0.0f)) return false;

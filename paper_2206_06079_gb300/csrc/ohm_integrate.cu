@@ -96,12 +96,17 @@ __global__ void __launch_bounds__(kBlock, 4) k_prepare_tsdf(DeviceMap m, CallArg
   prepare_tsdf_ray(m, args, i, i < args.n);
 }
 
-__global__ void __launch_bounds__(kBlock) k_tsdf_walk(DeviceMap m, long long n) {
+// Compiled for 4 blocks per SM, which the launch counts on.
+__global__ void __launch_bounds__(kBlock, 4) k_tsdf_walk(DeviceMap m, long long n) {
   chain_enter();
   if (latched(m)) return;
+  __shared__ uint32_t tab[8 * kBlock];
+  __shared__ uint32_t acc[2 * kBlock];
+  acc[threadIdx.x] = acc[kBlock + threadIdx.x] = 0;
+  __syncthreads();
   // whole warps iterate together (the walk is warp-collective)
   const long long np = (n + 31) & ~31LL;
-  OHM_GRID_STRIDE(i, np) tsdf_walk_ray(m, i, i < n);
+  OHM_GRID_STRIDE(i, np) tsdf_walk_ray(m, i, i < n, tab + threadIdx.x, acc + 2 * (threadIdx.x & ~31u));
 }
 
 __global__ void __launch_bounds__(kBlock) k_tsdf_apply(DeviceMap m) {
