@@ -195,19 +195,32 @@ __global__ void __launch_bounds__(kBlock) k_query(DeviceMap m, const float* pts,
         s[2 * k + 1] = p.y;
       }
       if (s[0] > 0) {
-        const double cnt = (double)s[0];
+        // In double, with one reciprocal for the nine quotients (a rounding
+        // or two of 2^-53 more each, far below the float outputs') and the
+        // exact numerators of the covariance in 64 bits where they fit:
+        // n Sxx <= n^2 2^(2F) < 2^62.  A double instruction takes a warp 64
+        // cycles of a scheduler; nine divisions and six 128-bit conversions
+        // made this 18.5 us for 20,000 points; 10.3 us this way.
+        const double cnt = (double)s[0], inv = 1.0 / cnt;
         const double cell = m.voxel_size / (double)(1LL << F);
         out[0] = (float)cnt;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
           const double corner = (double)((long long)v[k] * (1LL << F));
-          out[1 + k] = (float)(m.origin[k] + (corner + (double)s[1 + k] / cnt) * cell);
+          out[1 + k] = (float)(m.origin[k] + (corner + (double)s[1 + k] * inv) * cell);
         }
         const int pa[6] = {0, 0, 0, 1, 1, 2}, pb[6] = {0, 1, 2, 1, 2, 2};
+        const double scale = inv * cell, scale2 = scale * scale;
+        if (s[0] < (1LL << (31 - F))) {
 #pragma unroll
-        for (int k = 0; k < 6; ++k) {
-          const __int128 num = (__int128)s[0] * s[4 + k] - (__int128)s[1 + pa[k]] * s[1 + pb[k]];
-          out[4 + k] = (float)((double)num / (cnt * cnt) * cell * cell);
+          for (int k = 0; k < 6; ++k)
+            out[4 + k] = (float)((double)(s[0] * s[4 + k] - s[1 + pa[k]] * s[1 + pb[k]]) * scale2);
+        } else {
+#pragma unroll 1
+          for (int k = 0; k < 6; ++k) {
+            const __int128 num = (__int128)s[0] * s[4 + k] - (__int128)s[1 + pa[k]] * s[1 + pb[k]];
+            out[4 + k] = (float)((double)num * scale2);
+          }
         }
       }
     }
