@@ -584,9 +584,12 @@ static __device__ __noinline__ int32_t find_neighbour_rare(const DeviceMap& m, c
                                       idx, (r.flags >> kRaySignShift) & 7));
 }
 
-// Voxels per batch of the miss walk, and the blocks per SM it is compiled for.
+// Voxels per batch of the miss walk, and the blocks per SM it is compiled for
+// (batches of 3 / 4 / 5 / 6 on a mapped 131,072-ray tunnel scan: 73.6 / 73.0 / 69.7 /
+// 77 us: a segment of about 24 voxels takes five batches of 5 with the least left
+// over; 6 spills).
 #ifndef OHM_FAST_BATCH
-#define OHM_FAST_BATCH 4
+#define OHM_FAST_BATCH 5
 #endif
 #ifndef OHM_FAST_MIN_BLOCKS
 #define OHM_FAST_MIN_BLOCKS 4
@@ -836,9 +839,9 @@ __device__ __forceinline__ void piece_fill(const DeviceMap& m, const RayRec* rp,
 // and the code is kept small, one copy of the stepping: a software pipeline
 // of two batches and a second form that reads the floats directly were slower
 // by what they add to the instruction cache and the registers.
-// Measured (131,072-ray tunnel scan, 0.1 m, 865 k segments): 123.5 -> 72.4 us in
-// a mapped tunnel, 164 -> 154 us in unknown space; 262,144 rays at 0.05 m
-// 308 -> 162 us; outdoor scans into half-known space 144 -> 104 us.
+// Measured (131,072-ray tunnel scan, 0.1 m, 865 k segments): 123.5 -> 69.7 us in
+// a mapped tunnel, 164 -> 148 us in unknown space; 262,144 rays at 0.05 m
+// 308 -> 157 us; outdoor scans into half-known space 144 -> 101 us.
 template <bool kOcc, bool kCounts, bool kCas, bool kDecay>
 __device__ __forceinline__ void walk_segments(const DeviceMap& m, bool has, int2 sg, WalkShared& sh,
                                               unsigned int& ops, const RayRec* prefetch = nullptr) {
@@ -898,7 +901,7 @@ __device__ __forceinline__ void walk_segments(const DeviceMap& m, bool has, int2
     int rounds = __reduce_max_sync(full, left > 0 ? left + kFastBatch - 1 : 0) / kFastBatch;
     uint32_t brick = ~mo, word = 0;  // the last voxel stepped; the word of the last brick
     for (; rounds > 0; --rounds) {
-      uint32_t at[kFastBatch], off[kFastBatch], v[kFastBatch], valid;
+      uint32_t at[kFastBatch], off[kFastBatch], v[kFastBatch] = {}, valid;
       piece_fill(m, rp, K, tab, w, mo, left, at, off, valid);
       if (kCounts || kDecay) {
         const int lane = threadIdx.x & 31;
@@ -960,27 +963,28 @@ __device__ __forceinline__ void walk_segments(const DeviceMap& m, bool has, int2
         continue;
       }
       // the words of the bricks entered, then the voxels not known to be saturated
-      uint32_t entered = 0, open = valid;
-#pragma unroll
-      for (int j = 0; j < kFastBatch; ++j) {
-        if (((at[j] ^ (j ? at[j - 1] : brick)) & ~31u) && ((valid >> j) & 1u)) {
-          entered |= 1u << j;
-          v[j] = sat[off[j] >> 5];
-        }
-      }
+      const uint32_t before = brick;
       brick = at[kFastBatch - 1];
 #pragma unroll
+      for (int j = 0; j < kFastBatch; ++j)
+        if (((at[j] ^ (j ? at[j - 1] : before)) & ~31u) && ((valid >> j) & 1u)) v[j] = sat[off[j] >> 5];
+      bool open[kFastBatch], some = false;
+#pragma unroll
       for (int j = 0; j < kFastBatch; ++j) {
-        if ((entered >> j) & 1u) word = v[j];
-        open &= ~(((word >> (off[j] & 31u)) & 1u) << j);
+        if ((at[j] ^ (j ? at[j - 1] : before)) & ~31u) word = v[j];
+        open[j] = ((valid >> j) & 1u) && !((word >> (off[j] & 31u)) & 1u);
+        some = some || open[j];
       }
-      if (__any_sync(full, open != 0)) {
+      if (__any_sync(full, some)) {
         const int wid = threadIdx.x >> 5;
-        if (open) {
-          uint32_t i = atomicAdd(&sh.n_open[wid], (uint32_t)__popc(open));
+        if (some) {
+          uint32_t n = 0;
+#pragma unroll
+          for (int j = 0; j < kFastBatch; ++j) n += open[j] ? 1u : 0u;
+          uint32_t i = atomicAdd(&sh.n_open[wid], n);
 #pragma unroll
           for (int j = 0; j < kFastBatch; ++j)
-            if ((open >> j) & 1u) sh.open[wid][i++] = off[j];
+            if (open[j]) sh.open[wid][i++] = off[j];
         }
         __syncwarp();
         if (sh.n_open[wid] >= kOpenRound) ops += drain_open(m, sh, kOpenRound);
