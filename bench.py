@@ -400,7 +400,7 @@ def run_ours(args):
             "gpu_launches": int(launches),
             "stages_ms": stage_ms,
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
-                         "frac": achieved / hbm, "traffic": traffic, "kernel": "k_walk_fast<1, 0, 0>",
+                         "frac": achieved / hbm, "traffic": traffic, "kernel": "k_walk_fast<4>",
                          "algorithmic_bytes_per_launch": algo_bytes, "avg_launch_ms": walk_avg_s * 1e3,
                          "peak_source": peak_src,
                          "duration_source": "events around the walk in a replay of the timed scan sequence "

@@ -297,7 +297,7 @@ ohm_status ohm_probe_rate(int32_t device, int32_t kind, int64_t units, int64_t o
 
 /* Kernel stages of an integrate call, for per-stage GPU timing. */
 typedef enum {
-  OHM_STAGE_BEGIN = 0,        /* rollback snapshot */
+  OHM_STAGE_BEGIN = 0,        /* no kernel of its own: the end kernel readies the next call's counters */
   OHM_STAGE_PREPARE = 1,      /* quantise, truncate, region allocation, segment table, NDT
                                  layer of each sample's region where the slot is known */
   OHM_STAGE_NDT_ALLOC = 2,    /* NDT layer allocation for the sample regions prepare left */
@@ -306,7 +306,8 @@ typedef enum {
   OHM_STAGE_HITS = 5,         /* sample updates and NDT moments (phase two) */
   OHM_STAGE_TSDF_WALK = 6,    /* TSDF band walk */
   OHM_STAGE_TSDF_APPLY = 7,   /* TSDF weighted average */
-  OHM_STAGE_END = 8,          /* rollback of a failed call */
+  OHM_STAGE_END = 8,          /* rollback of a failed call, rollback snapshot and counters of the
+                                 next call, status copy */
   OHM_STAGE_MEAN_APPLY = 9,   /* voxel-mean per-call update */
   OHM_STAGE_COUNT = 10
 } ohm_stage;

@@ -85,16 +85,6 @@ OHM_UNROLL
 #endif
 }
 
-// A ray kept as its two fixed-point end points (the allocation-free entry
-// point's record).
-struct __align__(16) EndpointRec {
-  long long a[3];
-  long long b[3];
-  unsigned long long inv;
-  int32_t flags;
-  int32_t nseg;
-};
-
 // Ray record written by the TSDF prepare kernel: the walk covers the band
 // [max(0, d - tau), d + tau] of the ray from the sensor to the sample.
 struct __align__(16) TsdfRec {
@@ -1079,26 +1069,6 @@ OHM_UNROLL
   if (c[1] > p.c[1]) w.sy = fma_rn((float)(c[1] - p.c[1]), w.uy, w.sy);
   if (c[2] > p.c[2]) w.sz = fma_rn((float)(c[2] - p.c[2]), w.uz, w.sz);
   w.mn = fminf(w.sx, fminf(w.sy, w.sz));
-}
-
-// ---------------------------------------------------------------------------
-// Warp-aggregated reservation: every lane of a full warp calls this together
-// with its own count (possibly 0); returns this lane's first index.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ unsigned long long warp_reserve(unsigned long long* counter, unsigned int count) {
-  const unsigned full = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
-  unsigned int incl = count;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    unsigned int t = __shfl_up_sync(full, incl, o);
-    if (lane >= o) incl += t;
-  }
-  const unsigned int total = __shfl_sync(full, incl, 31);
-  unsigned long long base = 0;
-  if (lane == 31 && total != 0) base = atomicAdd(counter, (unsigned long long)total);
-  base = __shfl_sync(full, base, 31);
-  return base + incl - count;
 }
 
 // ---------------------------------------------------------------------------
