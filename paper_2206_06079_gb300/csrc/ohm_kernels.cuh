@@ -37,13 +37,13 @@ __device__ __forceinline__ void chain_enter() {
 // stream drains, and wait in chain_enter() until that kernel has completed.
 // Where the attribute is refused the kernel is launched the ordinary way.
 template <typename... K, typename... A>
-inline void launch_chained(void (*kernel)(K...), unsigned grid, cudaStream_t stream, A... args) {
+inline void launch_chained_of(unsigned block, void (*kernel)(K...), unsigned grid, cudaStream_t stream, A... args) {
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(kBlock);
+  cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = 0;
   cfg.stream = stream;
   cfg.attrs = attr;
@@ -53,6 +53,11 @@ inline void launch_chained(void (*kernel)(K...), unsigned grid, cudaStream_t str
     cfg.numAttrs = 0;
     (void)cudaLaunchKernelEx(&cfg, kernel, args...);
   }
+}
+
+template <typename... K, typename... A>
+inline void launch_chained(void (*kernel)(K...), unsigned grid, cudaStream_t stream, A... args) {
+  launch_chained_of(kBlock, kernel, grid, stream, args...);
 }
 
 // Tells the compiler that a pointer read from a DeviceMap outside constant
