@@ -53,7 +53,7 @@ struct DepthFrame {
 // Rows in bands of 4 (the last may be lower), columns in tiles of 8, the
 // columns left over behind them.
 __device__ __forceinline__ long long tile_pixel(long long p, int width, int height) {
-  if ((long long)width * height >= (1LL << 31)) return p;  // row by row
+  if ((long long)width * height >= (1LL << 31) || width >= (1 << 28)) return p;  // row by row (32-bit indices)
   const int i = (int)p;
   const int band = i / (4 * width), rows = height - 4 * band < 4 ? height - 4 * band : 4;
   const int t = i - band * 4 * width, tiles = width / 8, in_tiles = tiles * 8 * rows;

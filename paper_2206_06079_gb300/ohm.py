@@ -328,7 +328,7 @@ class Map:
 
     @staticmethod
     def _frame_args(K, pose):
-        return (ctypes.c_double * 4)(*K), Map._pose_arg(pose)
+        return (ctypes.c_double * 4)(*[float(v) for v in K]), Map._pose_arg(pose)
 
     def integrate_depth(self, depth, K, pose, z_min=0.3, z_max=6.0, stream=None, sync=True):
         """Integrate a z-depth image (CUDA float32 tensor, height x width) seen
