@@ -156,7 +156,7 @@ struct DeviceMap {
   float* grad;                   // [max_regions][32768] adjoint weights, allocated by the first backward call
   float* ndt_grad;               // [max_ndt][32768][9] NDT adjoint weights, allocated by the first NDT backward call
   int32_t* status;
-  int32_t* host_status;          // pinned host word: the status as the last finished call left it
+  int32_t* host_status;          // pinned host word: status of a call that failed, zero until then
   CallCounters* calls;
   // region cache (Sec. III-A: regions move between device and host memory)
   int32_t* stamp;                // [max_regions] seq of the last call that touched the region

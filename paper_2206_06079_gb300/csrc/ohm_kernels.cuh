@@ -306,15 +306,30 @@ __device__ __forceinline__ void snapshot_pool(const DeviceMap& m) {
 // and stand ready for the next call.  A failed call keeps its sequence number
 // and its rollback point, which the rollback (running beside this) reads.
 // Doing this here saves a kernel at the start of every call, about 3 us of a
-// small scan and one launch.
+// small scan and one launch.  One thread's latency bounds it, so every load
+// goes out before the first store, and the host's word, which ohm_map_sync
+// reads (and zeroes) without a copy of its own, is written after a failure
+// only.
 __device__ __forceinline__ void finish_call(const DeviceMap& m) {
   CallCounters* c = m.calls;
-  c->last.segments = c->segments;
-  c->last.visits = c->visits;
-  c->last.touched = c->touched;
-  c->last.atomics = c->atomics;
-  c->last.restores = c->restores;
-  c->total_visits += c->visits;
+  const auto segments = c->segments;
+  const auto visits = c->visits;
+  const auto touched = c->touched;
+  const auto atomics = c->atomics;
+  const auto restores = c->restores;
+  const auto total = c->total_visits;
+  const auto seq = c->seq;
+  const auto regions = *m.region_count;
+  const auto ndt_blocks = *m.ndt_count;
+  const auto free_used = m.free_info[1];
+  const auto ndt_free_used = m.free_info[3];
+  const int32_t status = *(volatile int32_t*)m.status;
+  c->last.segments = segments;
+  c->last.visits = visits;
+  c->last.touched = touched;
+  c->last.atomics = atomics;
+  c->last.restores = restores;
+  c->total_visits = total + visits;
   c->segments = 0;
   c->visits = 0;
   c->touched = 0;
@@ -322,13 +337,15 @@ __device__ __forceinline__ void finish_call(const DeviceMap& m) {
   c->restores = 0;
   c->ndt_pending = 0;
   c->mean_touched = 0;
-  const int32_t status = *(volatile int32_t*)m.status;
   if (status == 0) {
-    c->seq += 1;
-    snapshot_pool(m);
+    c->seq = seq + 1;
+    c->region_start = regions;
+    c->ndt_start = ndt_blocks;
+    c->free_used_start = free_used;
+    c->ndt_free_used_start = ndt_free_used;
+  } else {
+    *(volatile int32_t*)m.host_status = status;
   }
-  // read by ohm_map_sync without a copy of its own
-  *(volatile int32_t*)m.host_status = status;
 }
 
 // Fixed-point origin of the current call's rays where they share one: the
