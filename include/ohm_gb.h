@@ -393,8 +393,11 @@ ohm_status ohm_integrate_posed(ohm_map* map, const double* pose, const float* or
  * is recomputed, nothing is stored by the forward pass.  Call it before any
  * other integration into the map.  Needs the NDT layer and ndt_clear_below =
  * -INFINITY (OHM_ERR_UNSUPPORTED otherwise: sample clearing changes the
- * statistics discontinuously).  The first call allocates 36 bytes of weights
- * per voxel of the NDT pool.  All arrays are device memory except pose.
+ * statistics discontinuously).  The queries of one voxel are summed in double,
+ * so the results do not depend on the order of queries (grad_twist to a few
+ * 2^-53 per summand).  The first call allocates 4 bytes per voxel of the NDT
+ * pool; a call takes 72 bytes per query from a memory pool that the map keeps.
+ * All arrays are device memory except pose.
  * Returns once enqueued.  The paper has no counterpart. */
 ohm_status ohm_ndt_backward(ohm_map* map, const double* pose, const float* origins, int64_t n_origins,
                             const float* endpoints, const uint8_t* flags, int64_t n, const float* query_points,

@@ -290,43 +290,61 @@ __global__ void __launch_bounds__(kBlock) k_pose_rays(Pose34 P, CallArgs in, flo
   }
 }
 
-// Upstream weights of the NDT statistics per voxel: 9 floats (mean x y z,
-// covariance xx xy xz yy yz zz) per voxel of every NDT block.
-__device__ __forceinline__ float* ndt_grad_of(const DeviceMap& m, const float* p) {
+// Rows of upstream weights.  The queries that fall into one voxel share a row
+// of doubles, claimed by the first of them to arrive; `plane` holds the row
+// plus one of every voxel, 0 for none and between calls.  The sums are double
+// because the order in which queries arrive differs from run to run: in float
+// that moved a weight by 6e-8 of itself, which the double twist shows; in double
+// it is 1e-16.  A row per query, or per voxel where there are fewer of those.
+__device__ __forceinline__ long long claim_row(uint32_t* plane, long long off, long long row) {
+  uint32_t r = plane[off];
+  if (r == 0u) {
+    r = atomicCAS(plane + off, 0u, (uint32_t)row + 1u);
+    if (r == 0u) r = (uint32_t)row + 1u;
+  }
+  return (long long)r - 1;
+}
+
+// Index of the NDT voxel holding a point (block * 32768 + Morton index), -1:
+// outside the map or in a region without samples (nothing to differentiate).
+__device__ __forceinline__ long long ndt_point_offset(const DeviceMap& m, const float* p) {
   long long q[3];
   bool ok = true;
 #pragma unroll
   for (int k = 0; k < 3; ++k) ok = quantise_coord(m, p[k], k, &q[k]) && ok;
   ok = ok && in_extent(q, m.frac_bits);
-  if (!ok) return nullptr;
+  if (!ok) return -1;
   const int F = m.frac_bits;
   const int32_t vx = (int32_t)(q[0] >> F), vy = (int32_t)(q[1] >> F), vz = (int32_t)(q[2] >> F);
   const int32_t slot = region_slot_of(m, vx, vy, vz);
   const int32_t ns = slot < 0 ? -1 : m.ndt_slot[slot];
-  if (ns < 0) return nullptr;  // no samples in the region: nothing to differentiate
-  return m.ndt_grad + ((long long)ns * kRegionVoxels + local_morton(vx, vy, vz)) * 9;
+  return ns < 0 ? -1 : voxel_offset(ns, local_morton(vx, vy, vz));
 }
 
+// The upstream weights of a voxel (mean x y z, covariance xx xy xz yy yz zz),
+// summed over the queries it holds: a row of 9 doubles, added to for each
+// query point, or the voxels' rows forgotten (rows = null).
 __global__ void __launch_bounds__(kBlock) k_ndt_grad_scatter(DeviceMap m, const float* pts, const float* gmean,
-                                                             const float* gcov, long long n, int clear) {
+                                                             const float* gcov, long long n, double* rows,
+                                                             int by_voxel) {
   for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x) {
-    float* g = ndt_grad_of(m, pts + 3 * q);
-    if (!g) continue;
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-      if (clear)
-        g[k] = 0.f;
-      else
-        atomicAdd(g + k, k < 3 ? gmean[3 * q + k] : gcov[6 * q + k - 3]);
+    const long long off = ndt_point_offset(m, pts + 3 * q);
+    if (off < 0) continue;
+    if (!rows) {
+      m.ndt_grad_row[off] = 0u;
+      continue;
     }
+    double* g = rows + 9 * claim_row(m.ndt_grad_row, off, by_voxel ? off : q);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) atomicAdd(g + k, (double)(k < 3 ? gmean[3 * q + k] : gcov[6 * q + k - 3]));
   }
 }
 
 // Per ray of the frame (world rays in `a`, as integrated): the sample's voxel
 // by the quantisation and truncation of the forward pass, then dL/dp from the
 // voxel's moments and weights.
-__global__ void __launch_bounds__(kBlock) k_ndt_backward(DeviceMap m, CallArgs a, Pose34 P, float* grad_e,
-                                                         double* grad_twist) {
+__global__ void __launch_bounds__(kBlock) k_ndt_backward(DeviceMap m, CallArgs a, Pose34 P, const double* rows,
+                                                         float* grad_e, double* grad_twist) {
   __shared__ double red[kBlock / 32][6];
   const int F = m.frac_bits;
   const long long U = 1LL << F;
@@ -354,13 +372,13 @@ __global__ void __launch_bounds__(kBlock) k_ndt_backward(DeviceMap m, CallArgs a
         atomicOr(m.status, kStatusMissing);
       } else {
         const uint32_t mo = local_morton(v[0], v[1], v[2]);
-        const float* g = m.ndt_grad + ((long long)ns * kRegionVoxels + mo) * 9;
-        float w[9];
+        const uint32_t row = m.ndt_grad_row[voxel_offset(ns, mo)];  // 0: no query fell into the voxel
+        double w[9];
         bool any = false;
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
-          w[k] = g[k];
-          any = any || w[k] != 0.f;
+          w[k] = row ? rows[9LL * (row - 1u) + k] : 0.0;
+          any = any || w[k] != 0.0;
         }
         const long long* mom = ndt_moments(m, ns, mo);
         const double cnt = (double)mom[0];
@@ -372,7 +390,7 @@ __global__ void __launch_bounds__(kBlock) k_ndt_backward(DeviceMap m, CallArgs a
           // (G + G^T) d with G upper triangular from the packed xx xy xz yy yz zz
           const double Gs[3][3] = {{2.0 * w[3], w[4], w[5]}, {w[4], 2.0 * w[6], w[7]}, {w[5], w[7], 2.0 * w[8]}};
 #pragma unroll
-          for (int k = 0; k < 3; ++k) gp[k] = ((double)w[k] + Gs[k][0] * dv[0] + Gs[k][1] * dv[1] + Gs[k][2] * dv[2]) / cnt;
+          for (int k = 0; k < 3; ++k) gp[k] = (w[k] + Gs[k][0] * dv[0] + Gs[k][1] * dv[1] + Gs[k][2] * dv[2]) / cnt;
         }
       }
     }
@@ -470,6 +488,34 @@ cudaError_t frame_tables(ohm_map* map, DepthFrame* f, cudaStream_t s) {
   f->pxy = map->pxy;
   f->pxyf = reinterpret_cast<const float2*>(map->pxy + n);
   return cudaSuccess;
+}
+
+// Zeroed rows of `width` doubles for a backward call's queries (claim_row), one
+// per query or, where there are fewer, per voxel of the layer (*by_voxel).  They
+// come from the map's own memory pool in stream order and go back to it with
+// cudaFreeAsync, so calls on other streams and captured calls (whose graph then
+// holds the memory) never meet; the pool keeps its memory until the map goes.
+cudaError_t take_rows(ohm_map* map, long long n_query, long long voxels, int width, cudaStream_t s, double** rows,
+                      int* by_voxel) {
+  cudaError_t e = cudaSuccess;
+  if (!map->rows_pool) {
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = map->device;
+    e = cudaMemPoolCreate(&map->rows_pool, &props);
+    if (e != cudaSuccess) {
+      map->rows_pool = nullptr;
+      return e;
+    }
+    uint64_t keep = UINT64_MAX;
+    e = cudaMemPoolSetAttribute(map->rows_pool, cudaMemPoolAttrReleaseThreshold, &keep);
+  }
+  *by_voxel = n_query > voxels ? 1 : 0;
+  const size_t bytes = sizeof(double) * (size_t)width * (size_t)(*by_voxel ? voxels : n_query);
+  if (e == cudaSuccess) e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(rows), bytes, map->rows_pool, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(*rows, 0, bytes, s);
+  return e;
 }
 
 ohm_status afail(ohm_status code, const std::string& msg) {
@@ -661,16 +707,20 @@ ohm_status ohm_ndt_backward(ohm_map* map, const double* pose, const float* origi
   if (prev != map->device) cudaSetDevice(map->device);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   cudaError_t e = cudaSuccess;
-  if (!map->d.ndt_grad) {
-    // upstream weights per NDT voxel, allocated on the first backward call
-    const size_t bytes = sizeof(float) * 9 * (size_t)map->d.max_ndt * kRegionVoxels;
-    e = cudaMalloc(reinterpret_cast<void**>(&map->d.ndt_grad), bytes);
-    if (e == cudaSuccess) e = cudaMemset(map->d.ndt_grad, 0, bytes);
+  const long long voxels = (long long)map->d.max_ndt * kRegionVoxels;
+  if (!map->d.ndt_grad_row) {
+    // rows of upstream weights per NDT voxel, allocated on the first backward call
+    const size_t bytes = sizeof(uint32_t) * (size_t)voxels;
+    e = cudaMalloc(reinterpret_cast<void**>(&map->d.ndt_grad_row), bytes);
+    if (e == cudaSuccess) e = cudaMemset(map->d.ndt_grad_row, 0, bytes);
   }
   if (e == cudaSuccess) e = cudaMemsetAsync(grad_twist, 0, 6 * sizeof(double), s);
   const int qb = (int)(n_query > 0 ? ((n_query + kBlock - 1) / kBlock < 4096 ? (n_query + kBlock - 1) / kBlock : 4096) : 0);
+  double* rows = nullptr;
+  int by_voxel = 0;
+  if (e == cudaSuccess && qb) e = take_rows(map, n_query, voxels, 9, s, &rows, &by_voxel);
   if (e == cudaSuccess && qb) {
-    k_ndt_grad_scatter<<<qb, kBlock, 0, s>>>(map->d, query_points, grad_mean, grad_cov, n_query, 0);
+    k_ndt_grad_scatter<<<qb, kBlock, 0, s>>>(map->d, query_points, grad_mean, grad_cov, n_query, rows, by_voxel);
     map->launches += 1;
   }
   map->status_copied = false;  // k_ndt_backward can latch a failure
@@ -679,13 +729,17 @@ ohm_status ohm_ndt_backward(ohm_map* map, const double* pose, const float* origi
     e = stage_posed(map, P, origins, n_origins, endpoints, flags, n, s, &a);
     const int pb = (int)((n + kBlock - 1) / kBlock < 4096 ? (n + kBlock - 1) / kBlock : 4096);
     if (e == cudaSuccess) {
-      k_ndt_backward<<<pb, kBlock, 0, s>>>(map->d, a, P, grad_endpoints, grad_twist);
+      k_ndt_backward<<<pb, kBlock, 0, s>>>(map->d, a, P, rows, grad_endpoints, grad_twist);
       map->launches += 1;
     }
   }
   if (e == cudaSuccess && qb) {
-    k_ndt_grad_scatter<<<qb, kBlock, 0, s>>>(map->d, query_points, grad_mean, grad_cov, n_query, 1);
+    k_ndt_grad_scatter<<<qb, kBlock, 0, s>>>(map->d, query_points, grad_mean, grad_cov, n_query, nullptr, 0);
     map->launches += 1;
+  }
+  if (rows) {
+    const cudaError_t ef = cudaFreeAsync(rows, s);
+    if (e == cudaSuccess) e = ef;
   }
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e == cudaSuccess) note_work(map, s);

@@ -154,7 +154,8 @@ struct DeviceMap {
   uint32_t* tsdf_cnt;            // [max_regions][32768] per-call scratch, zero between calls
   long long* tsdf_sum;           // [max_regions][32768] per-call scratch, 2^-32 m units
   float* grad;                   // [max_regions][32768] adjoint weights, allocated by the first backward call
-  float* ndt_grad;               // [max_ndt][32768][9] NDT adjoint weights, allocated by the first NDT backward call
+  uint32_t* ndt_grad_row;        // [max_ndt][32768] row of a voxel's NDT adjoint weights plus one, zero between calls;
+                                 // allocated by the first NDT backward call
   int32_t* status;
   int32_t* host_status;          // pinned host word: status of a call that failed, zero until then
   CallCounters* calls;

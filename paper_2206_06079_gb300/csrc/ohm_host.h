@@ -40,6 +40,7 @@ struct ohm_map {
   bool status_copied;       // h_status[1] holds (once the stream has passed) what the device word holds
   ohm::CallCounters* h_calls;
   int32_t* h_count;
+  cudaMemPool_t rows_pool;  // working memory of the backward calls, made by the first of them
   long long launches;       // kernels launched by this map
   long long last_rays;      // rays of the last integrate call
   // per-stage event timing

@@ -1,0 +1,83 @@
+"""The adjoints' upstream weights: queries that share voxels are summed in
+double, so the gradients depend neither on the order in which the queries
+arrive nor on how the sums' rows are laid out (one per query, or one per voxel
+where there are more queries than voxels)."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2206_06079_gb300 import ohm, workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import __graft_entry__
+    __graft_entry__.build()
+    assert torch.cuda.is_available()
+
+
+def _cuda(x):
+    return torch.from_numpy(np.ascontiguousarray(x, np.float32)).cuda()
+
+
+def _ndt_frame(n_query, seed=0):
+    """2,048 rays whose samples lie in one region, and n_query queries in 300
+    of the sample voxels, with positive weights (no cancellation in a sum)."""
+    rng = np.random.default_rng(seed)
+    e = rng.uniform(0.3, 2.9, size=(2048, 3)).astype(np.float32)
+    q = e[rng.integers(0, 300, n_query)]
+    return e, q, np.abs(rng.normal(size=(n_query, 3))) + 0.1, np.abs(rng.normal(size=(n_query, 6))) + 0.1
+
+
+def _ndt_gradients(frame, order, max_ndt):
+    e, q, gm, gc = frame
+    P = np.eye(3, 4)
+    o = _cuda([[0.15, 0.15, 0.15]])
+    with ohm.Map(**W.tunnel_params(max_rays=2048, max_regions=64, max_ndt_regions=max_ndt)) as m:
+        m.integrate_posed(P, o, _cuda(e))
+        ge, gt = m.ndt_backward(P, o, _cuda(e), None, _cuda(q[order]), _cuda(gm[order]), _cuda(gc[order]))
+        m.sync()
+        return ge.cpu().numpy().astype(np.float64), gt.cpu().numpy()
+
+
+@pytest.mark.parametrize("n_query", [12000, 40000])
+def test_ndt_gradients_do_not_depend_on_the_order_of_queries(n_query):
+    frame = _ndt_frame(n_query)
+    rng = np.random.default_rng(1)
+    ge, gt = _ndt_gradients(frame, np.arange(n_query), 4)  # 131,072 voxels: a row per query
+    assert np.abs(gt).min() > 0
+    # a sum of k positive doubles is within k 2^-53 of itself in any order: the
+    # weights (at most n_query of a voxel), then the twist over the rays
+    e = frame[0].astype(np.float64)
+    size = np.abs(ge).sum(), (np.linalg.norm(e, axis=1) * np.linalg.norm(ge, axis=1)).sum()
+    tol = np.repeat(size, 3) * (n_query + len(e)) * 2.0 ** -52
+    for order, max_ndt in ((np.arange(n_query)[::-1], 4), (rng.permutation(n_query), 4), (rng.permutation(n_query), 1)):
+        ge2, gt2 = _ndt_gradients(frame, order, max_ndt)  # one block, 32,768 voxels: a row per voxel of 40,000 queries
+        assert (np.abs(gt2 - gt) <= tol).all(), (gt2 - gt, tol)
+        # float outputs of doubles that agree to 1e-11: adjacent floats at most
+        assert (np.abs(ge2 - ge) <= np.abs(ge) * 2.0 ** -23).all()
+
+
+def test_ndt_weights_replayed_from_a_graph():
+    """A captured backward holds its own rows: larger calls in between do not
+    reach them."""
+    small, large = _ndt_frame(500), _ndt_frame(30000, seed=3)
+    P = np.eye(3, 4)
+    o, e = _cuda([[0.15, 0.15, 0.15]]), _cuda(small[0])
+    a = [_cuda(x) for x in small[1:]]
+    b = [_cuda(x) for x in large[1:]]
+    with ohm.Map(**W.tunnel_params(max_rays=2048, max_regions=64, max_ndt_regions=4)) as m:
+        m.integrate_posed(P, o, e)
+        want = m.ndt_backward(P, o, e, None, *a)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            got = m.ndt_backward(P, o, e, None, *a)
+        for _ in range(2):
+            m.ndt_backward(P, o, e, None, *b)
+            g.replay()
+        torch.cuda.synchronize()
+        assert (got[0] - want[0]).abs().max() <= want[0].abs().max() * 2.0 ** -23
+        assert (got[1] - want[1]).abs().max() <= want[1].abs().max() * 2548 * 2.0 ** -52
