@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(kBlock, 2) k_tsdf_backward(DeviceMap m, DepthF
         for (int32_t left = ps.visits; left > 0;) {
           uint32_t at[kFastBatch], off[kFastBatch], valid;
           float G[kFastBatch];
-          piece_fill(m, &t.r, K, tab, w, mo, left, at, off, valid);
+          piece_fill<false>(m, &t.r, K, tab, w, mo, left, at, off, valid);
 #pragma unroll
           for (int j = 0; j < kFastBatch; ++j) G[j] = ((valid >> j) & 1u) ? m.grad[off[j]] : 0.f;
 #pragma unroll

@@ -759,6 +759,9 @@ __device__ __forceinline__ bool piece_regions(const DeviceMap& m, const PieceSta
 // kFastBatch steps of the local walk from `mo` (left: voxels of the piece not
 // yet stepped): sign-normalised Morton indices `at`, voxel offsets, and which of
 // them exist (`valid`).  rp, K: the ray and the piece's first dominant-axis step.
+// A voxel whose region is not in the map is dropped; kLatch: it also fails the
+// call, which inserted every region that it walks.
+template <bool kLatch = true>
 __device__ __forceinline__ void piece_fill(const DeviceMap& m, const RayRec* rp, int32_t K, uint32_t* tab, LWalker& w,
                                            uint32_t& mo, int32_t& left, uint32_t (&at)[kFastBatch],
                                            uint32_t (&off)[kFastBatch], uint32_t& valid) {
@@ -794,7 +797,7 @@ __device__ __forceinline__ void piece_fill(const DeviceMap& m, const RayRec* rp,
         if (e == kNoRegion) {
           const int32_t s = find_neighbour_rare(m, rp, K, idx);
           if (s < 0) {
-            atomicOr(m.status, kStatusMissing);
+            if (kLatch) atomicOr(m.status, kStatusMissing);
             valid &= ~(1u << j);
             continue;
           }
