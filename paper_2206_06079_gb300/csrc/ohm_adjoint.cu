@@ -189,20 +189,23 @@ __global__ void __launch_bounds__(kBlock, 2) k_tsdf_backward(DeviceMap m, DepthF
       const int M = (t.r.flags >> kRayAxisShift) & 3;
       const int32_t nmaj = M == 0 ? t.r.n[0] : (M == 1 ? t.r.n[1] : t.r.n[2]);
       float A = 0.f, B[3] = {0.f, 0.f, 0.f};
-      for (int32_t K = 0; K <= nmaj; K += kPieceSlots) {
+      // up to the first voxel whose region the map does not hold (moved to the
+      // host since the frame, or the frame was never integrated)
+      int32_t left = 0;
+      for (int32_t K = 0; K <= nmaj && left != kWalkEnded; K += kPieceSlots) {
         const int32_t Ke = K + kPieceSlots < nmaj + 1 ? K + kPieceSlots : nmaj + 1;
         PieceStart ps;
         LWalker w;
         uint32_t mo;
         piece_start(t.r, F, K, Ke, Ke == nmaj + 1, &ps, &w);
-        if (!piece_regions(m, ps, w, t.r.flags, tab, &mo)) break;  // not integrated: nothing to differentiate
+        if (!piece_regions<true>(m, ps, w, t.r.flags, tab, &mo)) break;
         int32_t rel[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) rel[k] = t.e[k] - ((ps.v[k] - t.r.v0[k]) << F);
-        for (int32_t left = ps.visits; left > 0;) {
+        for (left = ps.visits; left > 0;) {
           uint32_t at[kFastBatch], off[kFastBatch], valid;
           float G[kFastBatch];
-          piece_fill<false>(m, &t.r, K, tab, w, mo, left, at, off, valid);
+          piece_fill<true>(m, &t.r, K, tab, w, mo, left, at, off, valid);
 #pragma unroll
           for (int j = 0; j < kFastBatch; ++j) G[j] = ((valid >> j) & 1u) ? m.grad[off[j]] : 0.f;
 #pragma unroll

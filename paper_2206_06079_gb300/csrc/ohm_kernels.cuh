@@ -723,7 +723,8 @@ __device__ __forceinline__ unsigned int drain_open(const DeviceMap& m, WalkShare
 
 // Look up the regions of a piece and fill its column of the table; *mo becomes
 // the sign-normalised index of its first voxel.  False if its first or last
-// region is not in the map.
+// region is not in the map (kPartial: its first only).
+template <bool kPartial = false>
 __device__ __forceinline__ bool piece_regions(const DeviceMap& m, const PieceStart& p, const LWalker& w, int32_t flags,
                                               uint32_t* tab, uint32_t* mo) {
   const uint32_t neg = morton_neg(flags);
@@ -737,8 +738,8 @@ __device__ __forceinline__ bool piece_regions(const DeviceMap& m, const PieceSta
 #pragma unroll
   for (int i = 1; i < 8; ++i) tab[i * kBlock] = kNoRegion;
   tab[0] = region_entry(slot, neg, 0);
-  tab[idx * kBlock] = region_entry(slotE, neg, idx);
-  if (slot < 0 || slotE < 0) return false;
+  tab[idx * kBlock] = kPartial && slotE < 0 ? kNoRegion : region_entry(slotE, neg, idx);
+  if (slot < 0 || (!kPartial && slotE < 0)) return false;
   if (idx & (idx - 1u)) {  // two or three boundaries: the regions between
     // the parameter at which the piece leaves its first region, per axis it does
     const float o0 = (idx & 1u) ? w.sx + (float)((signs & 1) ? p.v[0] & 31 : ~p.v[0] & 31) * w.ux : INFINITY;
@@ -759,9 +760,11 @@ __device__ __forceinline__ bool piece_regions(const DeviceMap& m, const PieceSta
 // kFastBatch steps of the local walk from `mo` (left: voxels of the piece not
 // yet stepped): sign-normalised Morton indices `at`, voxel offsets, and which of
 // them exist (`valid`).  rp, K: the ray and the piece's first dominant-axis step.
-// A voxel whose region is not in the map is dropped; kLatch: it also fails the
-// call, which inserted every region that it walks.
-template <bool kLatch = true>
+// A voxel whose region is not in the map fails the call, which inserted every
+// region that it walks; kPartial (a map that may lack some): it ends the walk,
+// left = kWalkEnded.
+constexpr int32_t kWalkEnded = INT_MIN;
+template <bool kPartial = false>
 __device__ __forceinline__ void piece_fill(const DeviceMap& m, const RayRec* rp, int32_t K, uint32_t* tab, LWalker& w,
                                            uint32_t& mo, int32_t& left, uint32_t (&at)[kFastBatch],
                                            uint32_t (&off)[kFastBatch], uint32_t& valid) {
@@ -797,7 +800,12 @@ __device__ __forceinline__ void piece_fill(const DeviceMap& m, const RayRec* rp,
         if (e == kNoRegion) {
           const int32_t s = find_neighbour_rare(m, rp, K, idx);
           if (s < 0) {
-            if (kLatch) atomicOr(m.status, kStatusMissing);
+            if (kPartial) {
+              valid &= (1u << j) - 1u;
+              left = kWalkEnded;
+              return;
+            }
+            atomicOr(m.status, kStatusMissing);
             valid &= ~(1u << j);
             continue;
           }

@@ -99,3 +99,45 @@ def test_missing_regions_leave_the_map_usable():
     before = m.query(_cuda(end), tsdf=True)["tsdf"][0, 1].item()
     m.integrate(_cuda(end - [0.5, 0, 0]), _cuda(end))
     assert m.query(_cuda(end), tsdf=True)["tsdf"][0, 1].item() == before + 1
+
+
+@pytest.mark.parametrize("kept", list(KEPT))
+def test_gradient_up_to_the_first_missing_region(kept):
+    """Each ray's band counts up to its first voxel in a missing region, as
+    the sum over its unclamped voxels in float64 (1e-3 relative: the kernel's s
+    and chain rule are float32)."""
+    m, depth, K, pose = _map_with(KEPT[kept])
+    bands, o, e, pt = _bands(depth, K, pose)
+    vox, g = _queries(bands)
+    gd, gt = m.tsdf_backward(_cuda(depth), K, pose, _cuda((vox + 0.5) * VOXEL), _cuda(g))
+    m.sync()
+    weight = {tuple(v): float(x) for v, x in zip(vox.tolist(), g)}
+    held = set(KEPT[kept])
+    at = {}
+    for b in bands:
+        for v in ([] if b is None else b[0].tolist()):
+            at[tuple(v)] = None
+    w = m.query(_cuda((np.array(list(at)) + 0.5) * VOXEL), tsdf=True)["tsdf"][:, 1].cpu().numpy().astype(np.float64)
+    at = dict(zip(at, w))
+    ge, go = np.zeros((len(e), 3)), np.zeros(3)
+    cut = 0
+    for j, b in enumerate(bands):
+        if b is None:
+            continue
+        A, B = 0.0, np.zeros(3)
+        for v, s, r in zip(b[0].tolist(), b[1], b[2]):
+            if tuple(c >> 5 for c in v) not in held:
+                cut += 1
+                break
+            if abs(s) < TAU and tuple(v) in weight:
+                wv = weight[tuple(v)] / at[tuple(v)]
+                A += wv
+                B += wv * (r - s * b[3])
+        ge[j] = A * b[3] + B / b[4]
+        go -= B / b[4]
+    assert (cut > 0) == (kept != "all")
+    gz, twist = adjoint.chain_to_depth_and_twist(ge, go, e, o, pose[:, :3], pt)
+    gd = gd.cpu().numpy().reshape(-1).astype(np.float64)
+    assert np.abs(gz).max() > 0
+    assert (np.abs(gd - gz) <= 1e-3 * np.abs(gz) + 1e-6 * np.abs(gz).max()).all(), np.abs(gd - gz).max()
+    assert np.linalg.norm(gt.cpu().numpy() - twist) <= 1e-3 * np.linalg.norm(twist)
