@@ -736,11 +736,10 @@ ohm_status ohm_ndt_backward(ohm_map* map, const double* pose, const float* origi
       map->launches += 1;
     }
   }
-  if (e == cudaSuccess && qb) {
+  if (rows) {
+    // whatever else failed: no row may outlive its call in the plane
     k_ndt_grad_scatter<<<qb, kBlock, 0, s>>>(map->d, query_points, grad_mean, grad_cov, n_query, nullptr, 0);
     map->launches += 1;
-  }
-  if (rows) {
     const cudaError_t ef = cudaFreeAsync(rows, s);
     if (e == cudaSuccess) e = ef;
   }
