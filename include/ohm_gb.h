@@ -358,8 +358,11 @@ ohm_status ohm_integrate_depth(ohm_map* map, const float* depth, int32_t width, 
  * walk is recomputed, nothing is stored by the forward pass.  Call it before
  * any other integration into the map, with the same frame arguments as the
  * forward call, and with TSDF weights below tsdf_wmax.  All arrays are device
- * memory except intrinsics and pose.  The first call allocates a per-voxel
- * weight layer (4 bytes per pool voxel).  Returns once enqueued. */
+ * memory except intrinsics and pose.  The queries of one voxel are summed in
+ * double, so the results do not depend on the order of queries.  The walk of a
+ * band ends at the first voxel whose region the map does not hold.  The first
+ * call allocates 4 bytes per pool voxel; a call takes 8 bytes per query from a
+ * memory pool that the map keeps.  Returns once enqueued. */
 ohm_status ohm_tsdf_backward(ohm_map* map, const float* depth, int32_t width, int32_t height,
                              const double* intrinsics, const double* pose, double z_min, double z_max,
                              const float* query_points, const float* grad_query, int64_t n_query, float* grad_depth,

@@ -141,16 +141,33 @@ __device__ __forceinline__ long long point_offset(const DeviceMap& m, const floa
   return slot < 0 ? -1 : voxel_offset(slot, local_morton(vx, vy, vz));
 }
 
-// G(v) += g_q for each query point (clear = 0), or G(v) = 0 (clear = 1).
+// Rows of upstream weights.  The queries that fall into one voxel share a row
+// of doubles, claimed by the first of them to arrive; `plane` holds the row
+// plus one of every voxel, 0 for none and between calls.  The sums are double
+// because the order in which queries arrive differs from run to run: in float
+// that moved a weight by 6e-8 of itself, which the double twist shows; in double
+// it is 1e-16.  A row per query, or per voxel where there are fewer of those.
+__device__ __forceinline__ long long claim_row(uint32_t* plane, long long off, long long row) {
+  uint32_t r = plane[off];
+  if (r == 0u) {
+    r = atomicCAS(plane + off, 0u, (uint32_t)row + 1u);
+    if (r == 0u) r = (uint32_t)row + 1u;
+  }
+  return (long long)r - 1;
+}
+
+// The upstream weight G(v) of a voxel, the sum of g_q over the queries it
+// holds: a row of one double, added to for each query point, or the voxels'
+// rows forgotten (rows = null).
 __global__ void __launch_bounds__(kBlock) k_grad_scatter(DeviceMap m, const float* pts, const float* g, long long n,
-                                                         int clear) {
+                                                         double* rows, int by_voxel) {
   for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x) {
     const long long off = point_offset(m, pts + 3 * q);
     if (off < 0) continue;
-    if (clear)
-      m.grad[off] = 0.f;
+    if (!rows)
+      m.grad_row[off] = 0u;
     else
-      atomicAdd(m.grad + off, g[q]);
+      atomicAdd(rows + claim_row(m.grad_row, off, by_voxel ? off : q), (double)g[q]);
   }
 }
 
@@ -163,8 +180,8 @@ __device__ __forceinline__ double warp_sum(double v) {
 // Compiled for 2 blocks per SM (128 registers; 184 unbounded, which fits one;
 // 3 and 4 blocks: no difference).  640 x 480 frame with 20,000 queries: 121 us with
 // the double back-projection and the 64-bit walker, row by row; 100 us now.
-__global__ void __launch_bounds__(kBlock, 2) k_tsdf_backward(DeviceMap m, DepthFrame f, float* grad_depth,
-                                                          double* grad_twist) {
+__global__ void __launch_bounds__(kBlock, 2) k_tsdf_backward(DeviceMap m, DepthFrame f, const double* rows,
+                                                          float* grad_depth, double* grad_twist) {
   __shared__ double red[kBlock / 32][6];
   __shared__ uint32_t tabs[8 * kBlock];
   uint32_t* const tab = tabs + threadIdx.x;
@@ -203,11 +220,13 @@ __global__ void __launch_bounds__(kBlock, 2) k_tsdf_backward(DeviceMap m, DepthF
 #pragma unroll
         for (int k = 0; k < 3; ++k) rel[k] = t.e[k] - ((ps.v[k] - t.r.v0[k]) << F);
         for (left = ps.visits; left > 0;) {
-          uint32_t at[kFastBatch], off[kFastBatch], valid;
+          uint32_t at[kFastBatch], off[kFastBatch], row[kFastBatch], valid;
           float G[kFastBatch];
           piece_fill<true>(m, &t.r, K, tab, w, mo, left, at, off, valid);
 #pragma unroll
-          for (int j = 0; j < kFastBatch; ++j) G[j] = ((valid >> j) & 1u) ? m.grad[off[j]] : 0.f;
+          for (int j = 0; j < kFastBatch; ++j) row[j] = ((valid >> j) & 1u) ? m.grad_row[off[j]] : 0u;
+#pragma unroll
+          for (int j = 0; j < kFastBatch; ++j) G[j] = row[j] ? (float)rows[row[j] - 1u] : 0.f;
 #pragma unroll
           for (int j = 0; j < kFastBatch; ++j) {
             if (G[j] != 0.f) {
@@ -291,21 +310,6 @@ __global__ void __launch_bounds__(kBlock) k_pose_rays(Pose34 P, CallArgs in, flo
     if (i < in.n_origins) pose_point(P, in.origins + 3 * i, origins + 3 * i);
     flags[i] = in.flags ? in.flags[i] : 0;
   }
-}
-
-// Rows of upstream weights.  The queries that fall into one voxel share a row
-// of doubles, claimed by the first of them to arrive; `plane` holds the row
-// plus one of every voxel, 0 for none and between calls.  The sums are double
-// because the order in which queries arrive differs from run to run: in float
-// that moved a weight by 6e-8 of itself, which the double twist shows; in double
-// it is 1e-16.  A row per query, or per voxel where there are fewer of those.
-__device__ __forceinline__ long long claim_row(uint32_t* plane, long long off, long long row) {
-  uint32_t r = plane[off];
-  if (r == 0u) {
-    r = atomicCAS(plane + off, 0u, (uint32_t)row + 1u);
-    if (r == 0u) r = (uint32_t)row + 1u;
-  }
-  return (long long)r - 1;
 }
 
 // Index of the NDT voxel holding a point (block * 32768 + Morton index), -1:
@@ -599,27 +603,34 @@ ohm_status ohm_tsdf_backward(ohm_map* map, const float* depth, int32_t width, in
   if (prev != map->device) cudaSetDevice(map->device);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   cudaError_t e = cudaSuccess;
-  if (!map->d.grad) {
-    // per-voxel gradient weights, allocated on the first backward call
-    e = cudaMalloc(reinterpret_cast<void**>(&map->d.grad), sizeof(float) * (size_t)map->p.max_regions * kRegionVoxels);
-    if (e == cudaSuccess) e = cudaMemset(map->d.grad, 0, sizeof(float) * (size_t)map->p.max_regions * kRegionVoxels);
+  const long long voxels = (long long)map->p.max_regions * kRegionVoxels;
+  if (!map->d.grad_row) {
+    // rows of upstream weights per voxel, allocated on the first backward call
+    e = cudaMalloc(reinterpret_cast<void**>(&map->d.grad_row), sizeof(uint32_t) * (size_t)voxels);
+    if (e == cudaSuccess) e = cudaMemset(map->d.grad_row, 0, sizeof(uint32_t) * (size_t)voxels);
   }
   const long long n = (long long)width * height;
   const int qb = (int)(n_query > 0 ? ((n_query + kBlock - 1) / kBlock < 4096 ? (n_query + kBlock - 1) / kBlock : 4096) : 0);
   const int pb = (int)((n + kBlock - 1) / kBlock < 4096 ? (n + kBlock - 1) / kBlock : 4096);
   if (e == cudaSuccess) e = frame_tables(map, &f, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(grad_twist, 0, 6 * sizeof(double), s);
+  double* rows = nullptr;
+  int by_voxel = 0;
+  if (e == cudaSuccess && qb) e = take_rows(map, n_query, voxels, 1, s, &rows, &by_voxel);
   if (e == cudaSuccess && qb) {
-    k_grad_scatter<<<qb, kBlock, 0, s>>>(map->d, query_points, grad_query, n_query, 0);
+    k_grad_scatter<<<qb, kBlock, 0, s>>>(map->d, query_points, grad_query, n_query, rows, by_voxel);
     map->launches += 1;
   }
   if (e == cudaSuccess) {
-    k_tsdf_backward<<<pb, kBlock, 0, s>>>(map->d, f, grad_depth, grad_twist);
+    k_tsdf_backward<<<pb, kBlock, 0, s>>>(map->d, f, rows, grad_depth, grad_twist);
     map->launches += 1;
   }
-  if (e == cudaSuccess && qb) {
-    k_grad_scatter<<<qb, kBlock, 0, s>>>(map->d, query_points, grad_query, n_query, 1);
+  if (rows) {
+    // whatever else failed: no row may outlive its call in the plane
+    k_grad_scatter<<<qb, kBlock, 0, s>>>(map->d, query_points, grad_query, n_query, nullptr, 0);
     map->launches += 1;
+    const cudaError_t ef = cudaFreeAsync(rows, s);
+    if (e == cudaSuccess) e = ef;
   }
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e == cudaSuccess) note_work(map, s);

@@ -153,7 +153,8 @@ struct DeviceMap {
   float2* tsdf;                  // [max_regions][32768] (D, W)
   uint32_t* tsdf_cnt;            // [max_regions][32768] per-call scratch, zero between calls
   long long* tsdf_sum;           // [max_regions][32768] per-call scratch, 2^-32 m units
-  float* grad;                   // [max_regions][32768] adjoint weights, allocated by the first backward call
+  uint32_t* grad_row;            // [max_regions][32768] row of a voxel's TSDF adjoint weight plus one, zero between calls;
+                                 // allocated by the first backward call
   uint32_t* ndt_grad_row;        // [max_ndt][32768] row of a voxel's NDT adjoint weights plus one, zero between calls;
                                  // allocated by the first NDT backward call
   int32_t* status;

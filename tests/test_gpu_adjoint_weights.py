@@ -81,3 +81,35 @@ def test_ndt_weights_replayed_from_a_graph():
         torch.cuda.synchronize()
         assert (got[0] - want[0]).abs().max() <= want[0].abs().max() * 2.0 ** -23
         assert (got[1] - want[1]).abs().max() <= want[1].abs().max() * 2548 * 2.0 ** -52
+
+
+@pytest.mark.parametrize("n_query", [8000, 40000])
+def test_tsdf_gradients_do_not_depend_on_the_order_of_queries(n_query):
+    """A 32 x 24 frame onto a wall inside one region, queries in 150 band
+    voxels with positive weights."""
+    rng = np.random.default_rng(2)
+    w, h = 32, 24
+    K, pose = (60.0, 60.0, 15.5, 11.5), np.concatenate([np.eye(3), np.full((3, 1), 0.8)], 1)
+    pose[2, 3] = 0.25
+    depth = _cuda(0.7 + 0.02 * rng.random((h, w)))
+    vox = np.stack(np.meshgrid(np.arange(12, 20), np.arange(12, 20), np.arange(16, 22)), -1).reshape(-1, 3)[rng.permutation(384)[:150]]
+    pts = (vox + 0.5)[rng.integers(0, 150, n_query)] * 0.05
+    g = np.abs(rng.normal(size=n_query)) + 0.1
+
+    def gradients(order, max_regions):
+        with ohm.Map(**W.tsdf_params(max_rays=w * h, max_regions=max_regions)) as m:
+            m.integrate_depth(depth, K, pose)
+            assert m.region_count() == 1
+            gd, gt = m.tsdf_backward(depth, K, pose, _cuda(pts[order]), _cuda(g[order]))
+            m.sync()
+            return gd.cpu().numpy().astype(np.float64), gt.cpu().numpy()
+
+    gd, gt = gradients(np.arange(n_query), 2)  # 65,536 voxels: a row per query
+    assert np.abs(gd).max() > 0
+    for order, regions in ((np.arange(n_query)[::-1], 2), (rng.permutation(n_query), 2), (rng.permutation(n_query), 1)):
+        gd2, gt2 = gradients(order, regions)  # 32,768 voxels: a row per voxel of 40,000 queries
+        # each weight enters as the float nearest to its double sum, which the
+        # order moves by n_query 2^-53 of itself: for 150 voxels no float changes
+        assert np.array_equal(gd2, gd)
+        # the pixels' float contributions (under 2 m from the origin) summed in double
+        assert np.abs(gt2 - gt).max() <= 4 * np.abs(gd).sum() * gd.size * 2.0 ** -52
