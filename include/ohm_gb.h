@@ -361,8 +361,8 @@ ohm_status ohm_integrate_depth(ohm_map* map, const float* depth, int32_t width, 
  * memory except intrinsics and pose.  The queries of one voxel are summed in
  * double, so the results do not depend on the order of queries.  The walk of a
  * band ends at the first voxel whose region the map does not hold.  The first
- * call allocates 4 bytes per pool voxel; a call takes 8 bytes per query from a
- * memory pool that the map keeps.  Returns once enqueued. */
+ * call allocates 4 bytes per pool voxel, and a call with more queries than any
+ * before 8 bytes per query.  Returns once enqueued. */
 ohm_status ohm_tsdf_backward(ohm_map* map, const float* depth, int32_t width, int32_t height,
                              const double* intrinsics, const double* pose, double z_min, double z_max,
                              const float* query_points, const float* grad_query, int64_t n_query, float* grad_depth,
@@ -399,7 +399,7 @@ ohm_status ohm_integrate_posed(ohm_map* map, const double* pose, const float* or
  * statistics discontinuously).  The queries of one voxel are summed in double,
  * so the results do not depend on the order of queries (grad_twist to a few
  * 2^-53 per summand).  The first call allocates 4 bytes per voxel of the NDT
- * pool; a call takes 72 bytes per query from a memory pool that the map keeps.
+ * pool, and a call with more queries than any before 72 bytes per query.
  * All arrays are device memory except pose.
  * Returns once enqueued.  The paper has no counterpart. */
 ohm_status ohm_ndt_backward(ohm_map* map, const double* pose, const float* origins, int64_t n_origins,

@@ -25,6 +25,7 @@
 // p (relative to its corner) and d = p_j - S / n,
 //   dL/dp_j = (1 / n) [ gm + (G + G^T) d ],  G = upper-triangular(gc),
 // then dL/de_sensor = R^T dL/dp_j and the twist as for the TSDF.
+#include <algorithm>
 #include <cstring>
 #include <string>
 #include <vector>
@@ -157,17 +158,20 @@ __device__ __forceinline__ long long claim_row(uint32_t* plane, long long off, l
 }
 
 // The upstream weight G(v) of a voxel, the sum of g_q over the queries it
-// holds: a row of one double, added to for each query point, or the voxels'
-// rows forgotten (rows = null).
+// holds: a row of one double, added to for each query point, or (clear) zeroed
+// and forgotten.
 __global__ void __launch_bounds__(kBlock) k_grad_scatter(DeviceMap m, const float* pts, const float* g, long long n,
-                                                         double* rows, int by_voxel) {
+                                                         double* rows, int by_voxel, int clear) {
   for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x) {
     const long long off = point_offset(m, pts + 3 * q);
     if (off < 0) continue;
-    if (!rows)
+    if (clear) {
+      const uint32_t row = m.grad_row[off];  // 0: another query of the voxel was here
+      if (row) rows[row - 1u] = 0.0;
       m.grad_row[off] = 0u;
-    else
+    } else {
       atomicAdd(rows + claim_row(m.grad_row, off, by_voxel ? off : q), (double)g[q]);
+    }
   }
 }
 
@@ -330,14 +334,18 @@ __device__ __forceinline__ long long ndt_point_offset(const DeviceMap& m, const 
 
 // The upstream weights of a voxel (mean x y z, covariance xx xy xz yy yz zz),
 // summed over the queries it holds: a row of 9 doubles, added to for each
-// query point, or the voxels' rows forgotten (rows = null).
+// query point, or (clear) zeroed and forgotten.
 __global__ void __launch_bounds__(kBlock) k_ndt_grad_scatter(DeviceMap m, const float* pts, const float* gmean,
                                                              const float* gcov, long long n, double* rows,
-                                                             int by_voxel) {
+                                                             int by_voxel, int clear) {
   for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x) {
     const long long off = ndt_point_offset(m, pts + 3 * q);
     if (off < 0) continue;
-    if (!rows) {
+    if (clear) {
+      const uint32_t row = m.ndt_grad_row[off];  // 0: another query of the voxel was here
+#pragma unroll
+      for (int k = 0; k < 9; ++k)
+        if (row) rows[9LL * (row - 1u) + k] = 0.0;
       m.ndt_grad_row[off] = 0u;
       continue;
     }
@@ -498,32 +506,49 @@ cudaError_t frame_tables(ohm_map* map, DepthFrame* f, cudaStream_t s) {
 }
 
 // Zeroed rows of `width` doubles for a backward call's queries (claim_row), one
-// per query or, where there are fewer, per voxel of the layer (*by_voxel).  They
-// come from the map's own memory pool in stream order and go back to it with
-// cudaFreeAsync, so calls on other streams and captured calls (whose graph then
-// holds the memory) never meet; the pool keeps its memory until the map goes.
-cudaError_t take_rows(ohm_map* map, long long n_query, long long voxels, int width, cudaStream_t s, double** rows,
-                      int* by_voxel) {
-  cudaError_t e = cudaSuccess;
-  if (!map->rows_pool) {
-    cudaMemPoolProps props = {};
-    props.allocType = cudaMemAllocationTypePinned;
-    props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = map->device;
-    e = cudaMemPoolCreate(&map->rows_pool, &props);
+// per query or, where there are fewer, per voxel of the layer.  The buffer stays
+// with the map and the clearing pass zeroes what the call used, so that a call
+// costs no allocation and no fill (a pool allocation and a fill for each call
+// took 12 to 30 us of 510).  It grows by doubling; a captured call that finds it
+// too small takes memory that its graph then holds (`own`).
+struct Rows {
+  double* p = nullptr;
+  int by_voxel = 0;
+  bool own = false;
+};
+cudaError_t take_rows(ohm_map* map, long long n_query, long long voxels, int width, cudaStream_t s, Rows* r) {
+  r->by_voxel = n_query > voxels ? 1 : 0;
+  const long long need = width * (r->by_voxel ? voxels : n_query);
+  if (need <= map->rows_cap) {
+    r->p = map->rows.back();
+    return cudaSuccess;
+  }
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  cudaError_t e = cudaStreamIsCapturing(s, &capture);
+  if (e != cudaSuccess) return e;
+  double* p = nullptr;
+  long long cap = need;
+  if (capture != cudaStreamCaptureStatusNone) {
+    e = cudaMallocAsync(reinterpret_cast<void**>(&p), sizeof(double) * (size_t)need, s);
+    r->own = e == cudaSuccess;
+  } else {
+    cap = std::max(need, std::max(2 * map->rows_cap, 1LL << 16));
+    e = cudaMalloc(reinterpret_cast<void**>(&p), sizeof(double) * (size_t)cap);
+  }
+  if (e != cudaSuccess) return e;
+  e = cudaMemsetAsync(p, 0, sizeof(double) * (size_t)cap, s);
+  if (!r->own) {
     if (e != cudaSuccess) {
-      map->rows_pool = nullptr;
+      cudaFree(p);
       return e;
     }
-    uint64_t keep = UINT64_MAX;
-    e = cudaMemPoolSetAttribute(map->rows_pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    map->rows.push_back(p);
+    map->rows_cap = cap;
   }
-  *by_voxel = n_query > voxels ? 1 : 0;
-  const size_t bytes = sizeof(double) * (size_t)width * (size_t)(*by_voxel ? voxels : n_query);
-  if (e == cudaSuccess) e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(rows), bytes, map->rows_pool, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(*rows, 0, bytes, s);
+  r->p = p;
   return e;
 }
+cudaError_t give_rows(const Rows& r, cudaStream_t s) { return r.own ? cudaFreeAsync(r.p, s) : cudaSuccess; }
 
 ohm_status afail(ohm_status code, const std::string& msg) {
   set_last_error(msg);
@@ -607,29 +632,28 @@ ohm_status ohm_tsdf_backward(ohm_map* map, const float* depth, int32_t width, in
   if (!map->d.grad_row) {
     // rows of upstream weights per voxel, allocated on the first backward call
     e = cudaMalloc(reinterpret_cast<void**>(&map->d.grad_row), sizeof(uint32_t) * (size_t)voxels);
-    if (e == cudaSuccess) e = cudaMemset(map->d.grad_row, 0, sizeof(uint32_t) * (size_t)voxels);
+    if (e == cudaSuccess) e = cudaMemsetAsync(map->d.grad_row, 0, sizeof(uint32_t) * (size_t)voxels, s);
   }
   const long long n = (long long)width * height;
   const int qb = (int)(n_query > 0 ? ((n_query + kBlock - 1) / kBlock < 4096 ? (n_query + kBlock - 1) / kBlock : 4096) : 0);
   const int pb = (int)((n + kBlock - 1) / kBlock < 4096 ? (n + kBlock - 1) / kBlock : 4096);
   if (e == cudaSuccess) e = frame_tables(map, &f, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(grad_twist, 0, 6 * sizeof(double), s);
-  double* rows = nullptr;
-  int by_voxel = 0;
-  if (e == cudaSuccess && qb) e = take_rows(map, n_query, voxels, 1, s, &rows, &by_voxel);
+  Rows rows;
+  if (e == cudaSuccess && qb) e = take_rows(map, n_query, voxels, 1, s, &rows);
   if (e == cudaSuccess && qb) {
-    k_grad_scatter<<<qb, kBlock, 0, s>>>(map->d, query_points, grad_query, n_query, rows, by_voxel);
+    k_grad_scatter<<<qb, kBlock, 0, s>>>(map->d, query_points, grad_query, n_query, rows.p, rows.by_voxel, 0);
     map->launches += 1;
   }
   if (e == cudaSuccess) {
-    k_tsdf_backward<<<pb, kBlock, 0, s>>>(map->d, f, rows, grad_depth, grad_twist);
+    k_tsdf_backward<<<pb, kBlock, 0, s>>>(map->d, f, rows.p, grad_depth, grad_twist);
     map->launches += 1;
   }
-  if (rows) {
+  if (rows.p) {
     // whatever else failed: no row may outlive its call in the plane
-    k_grad_scatter<<<qb, kBlock, 0, s>>>(map->d, query_points, grad_query, n_query, nullptr, 0);
+    k_grad_scatter<<<qb, kBlock, 0, s>>>(map->d, query_points, grad_query, n_query, rows.p, rows.by_voxel, 1);
     map->launches += 1;
-    const cudaError_t ef = cudaFreeAsync(rows, s);
+    const cudaError_t ef = give_rows(rows, s);
     if (e == cudaSuccess) e = ef;
   }
   if (e == cudaSuccess) e = cudaGetLastError();
@@ -726,15 +750,14 @@ ohm_status ohm_ndt_backward(ohm_map* map, const double* pose, const float* origi
     // rows of upstream weights per NDT voxel, allocated on the first backward call
     const size_t bytes = sizeof(uint32_t) * (size_t)voxels;
     e = cudaMalloc(reinterpret_cast<void**>(&map->d.ndt_grad_row), bytes);
-    if (e == cudaSuccess) e = cudaMemset(map->d.ndt_grad_row, 0, bytes);
+    if (e == cudaSuccess) e = cudaMemsetAsync(map->d.ndt_grad_row, 0, bytes, s);
   }
   if (e == cudaSuccess) e = cudaMemsetAsync(grad_twist, 0, 6 * sizeof(double), s);
   const int qb = (int)(n_query > 0 ? ((n_query + kBlock - 1) / kBlock < 4096 ? (n_query + kBlock - 1) / kBlock : 4096) : 0);
-  double* rows = nullptr;
-  int by_voxel = 0;
-  if (e == cudaSuccess && qb) e = take_rows(map, n_query, voxels, 9, s, &rows, &by_voxel);
+  Rows rows;
+  if (e == cudaSuccess && qb) e = take_rows(map, n_query, voxels, 9, s, &rows);
   if (e == cudaSuccess && qb) {
-    k_ndt_grad_scatter<<<qb, kBlock, 0, s>>>(map->d, query_points, grad_mean, grad_cov, n_query, rows, by_voxel);
+    k_ndt_grad_scatter<<<qb, kBlock, 0, s>>>(map->d, query_points, grad_mean, grad_cov, n_query, rows.p, rows.by_voxel, 0);
     map->launches += 1;
   }
   map->status_copied = false;  // k_ndt_backward can latch a failure
@@ -743,15 +766,15 @@ ohm_status ohm_ndt_backward(ohm_map* map, const double* pose, const float* origi
     e = stage_posed(map, P, origins, n_origins, endpoints, flags, n, s, &a);
     const int pb = (int)((n + kBlock - 1) / kBlock < 4096 ? (n + kBlock - 1) / kBlock : 4096);
     if (e == cudaSuccess) {
-      k_ndt_backward<<<pb, kBlock, 0, s>>>(map->d, a, P, rows, grad_endpoints, grad_twist);
+      k_ndt_backward<<<pb, kBlock, 0, s>>>(map->d, a, P, rows.p, grad_endpoints, grad_twist);
       map->launches += 1;
     }
   }
-  if (rows) {
+  if (rows.p) {
     // whatever else failed: no row may outlive its call in the plane
-    k_ndt_grad_scatter<<<qb, kBlock, 0, s>>>(map->d, query_points, grad_mean, grad_cov, n_query, nullptr, 0);
+    k_ndt_grad_scatter<<<qb, kBlock, 0, s>>>(map->d, query_points, grad_mean, grad_cov, n_query, rows.p, rows.by_voxel, 1);
     map->launches += 1;
-    const cudaError_t ef = cudaFreeAsync(rows, s);
+    const cudaError_t ef = give_rows(rows, s);
     if (e == cudaSuccess) e = ef;
   }
   if (e == cudaSuccess) e = cudaGetLastError();

@@ -89,7 +89,7 @@ void free_map(ohm_map* m) {
   ohm::destroy_host_store(m);
   for (void* p : ptrs)
     if (p) cudaFree(p);
-  if (m->rows_pool) cudaMemPoolDestroy(m->rows_pool);
+  for (double* r : m->rows) cudaFree(r);
   if (m->h_status) cudaFreeHost(m->h_status);
   if (m->h_calls) cudaFreeHost(m->h_calls);
   if (m->h_count) cudaFreeHost(m->h_count);

@@ -40,7 +40,10 @@ struct ohm_map {
   bool status_copied;       // h_status[1] holds (once the stream has passed) what the device word holds
   ohm::CallCounters* h_calls;
   int32_t* h_count;
-  cudaMemPool_t rows_pool;  // working memory of the backward calls, made by the first of them
+  // rows of the backward calls' weights (take_rows), all zero between calls: the
+  // last buffer is in use, smaller ones stay for graphs that captured them
+  std::vector<double*> rows;
+  long long rows_cap;       // doubles in the last of them
   long long launches;       // kernels launched by this map
   long long last_rays;      // rays of the last integrate call
   // per-stage event timing

@@ -60,27 +60,35 @@ def test_ndt_gradients_do_not_depend_on_the_order_of_queries(n_query):
         assert (np.abs(ge2 - ge) <= np.abs(ge) * 2.0 ** -23).all()
 
 
-def test_ndt_weights_replayed_from_a_graph():
-    """A captured backward holds its own rows: larger calls in between do not
-    reach them."""
-    small, large = _ndt_frame(500), _ndt_frame(30000, seed=3)
+@pytest.mark.parametrize("captured, between", [(500, 30000), (30000, 500), (30000, 60000)])
+def test_ndt_weights_replayed_from_a_graph(captured, between):
+    """A captured backward whose queries fit the rows that the map has, and
+    captured ones that do not; calls of other sizes, the map's rows growing,
+    in between."""
+    frame, other = _ndt_frame(captured), _ndt_frame(between, seed=3)
     P = np.eye(3, 4)
-    o, e = _cuda([[0.15, 0.15, 0.15]]), _cuda(small[0])
-    a = [_cuda(x) for x in small[1:]]
-    b = [_cuda(x) for x in large[1:]]
+    o, e = _cuda([[0.15, 0.15, 0.15]]), _cuda(frame[0])
+    a = [_cuda(x) for x in frame[1:]]
+    b = [_cuda(x) for x in other[1:]]
+    first = [x[:500] for x in a]
     with ohm.Map(**W.tunnel_params(max_rays=2048, max_regions=64, max_ndt_regions=4)) as m:
         m.integrate_posed(P, o, e)
-        want = m.ndt_backward(P, o, e, None, *a)
+        m.ndt_backward(P, o, e, None, *first)
         torch.cuda.synchronize()
         g = torch.cuda.CUDAGraph()
         with torch.cuda.graph(g):
             got = m.ndt_backward(P, o, e, None, *a)
+        want_b = m.ndt_backward(P, o, e, None, *b)
+        want = m.ndt_backward(P, o, e, None, *a)
         for _ in range(2):
-            m.ndt_backward(P, o, e, None, *b)
             g.replay()
+            got_b = m.ndt_backward(P, o, e, None, *b)
         torch.cuda.synchronize()
-        assert (got[0] - want[0]).abs().max() <= want[0].abs().max() * 2.0 ** -23
-        assert (got[1] - want[1]).abs().max() <= want[1].abs().max() * 2548 * 2.0 ** -52
+        for x, y in ((got, want), (got_b, want_b)):
+            n = captured + between + len(frame[0])
+            assert y[0].abs().max() > 0
+            assert (x[0] - y[0]).abs().max() <= y[0].abs().max() * 2.0 ** -23
+            assert (x[1] - y[1]).abs().max() <= y[1].abs().max() * n * 2.0 ** -52
 
 
 @pytest.mark.parametrize("n_query", [8000, 40000])
