@@ -8,14 +8,15 @@
 // allocator.  For them, ohm_count_rays_noalloc walks a ray set exactly like
 // ohm_integrate_rays and adds each ray's per-voxel hit and miss counts into
 // two uint32 arrays the caller owns.  Its per-call working memory (quantised
-// ray records) lives in one statically sized device array defined below, so
-// the call allocates nothing.
+// ray records and the length of each warp's rays) lives in one statically sized
+// device array defined below, so the call allocates nothing.
 //
 // That array is a file-scope __device__ variable: every GPU that loads this
 // library holds it (kNoAllocScratchBytes, 2 MB) until the process exits.
 // Every call shares it and writes the records it reads; calls whose work
 // overlaps on the GPU (different streams, no ordering between them) race on
 // it and must not be issued.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -31,7 +32,10 @@ constexpr long long kNoAllocMaxSegments = 4 * kNoAllocMaxRays;
 constexpr int kNoAllocBlock = 256;
 // dominant-axis slots of one thread's piece of a ray
 constexpr int kNoAllocSlots = 12;
-constexpr size_t kNoAllocScratchBytes = sizeof(RayRec) * kNoAllocMaxRays;
+// Layout of the static array: [ray records] [pieces of the longest ray of each warp].
+constexpr size_t kNoAllocRayBytes = sizeof(RayRec) * kNoAllocMaxRays;
+constexpr size_t kNoAllocScratchBytes = kNoAllocRayBytes + sizeof(int32_t) * (kNoAllocMaxRays / 32);
+static_assert(kNoAllocMaxRays % kNoAllocBlock == 0, "a length for each warp of the last block");
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
 
@@ -63,25 +67,27 @@ __device__ __forceinline__ bool na_in_extent(const long long q[3], int F) {
   return ok;
 }
 
-// Per ray: quantise, truncate to the maximum range.
-__global__ void __launch_bounds__(kNoAllocBlock) k_noalloc_prepare(CountGrid g, NoAllocArgs a, RayRec* rays) {
+// Per ray: quantise, truncate to the maximum range.  Per warp: the pieces of
+// its longest ray.
+__global__ void __launch_bounds__(kNoAllocBlock) k_noalloc_prepare(CountGrid g, NoAllocArgs a, RayRec* rays,
+                                                                   int32_t* warp_pieces) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int F = g.frac_bits;
-  if (i >= a.n) return;
   RayRec r;
   r.flags = 0;
   r.nseg = 0;
   r.inv = 0;
-  const long long oi = a.n_origins == 1 ? 0 : i;
+  const long long ei = i < a.n ? i : 0, oi = a.n_origins == 1 ? 0 : ei;
   long long qo[3], qe[3];
-  bool ok = true;
+  bool ok = i < a.n;
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    const float o = a.origins[3 * oi + k], e = a.endpoints[3 * i + k];
+    const float o = a.origins[3 * oi + k], e = a.endpoints[3 * ei + k];
     ok = ok && isfinite(o) && isfinite(e) && quantise(o, g.origin[k], g.scale, &qo[k]) &&
          quantise(e, g.origin[k], g.scale, &qe[k]);
   }
-  bool sample = !(a.flags && (a.flags[i] & kFlagNoReturn));
+  bool sample = !(a.flags && (a.flags[ei] & kFlagNoReturn));
+  int32_t pieces = 0;
   if (ok) {
     double d[3];
 #pragma unroll
@@ -103,8 +109,11 @@ __global__ void __launch_bounds__(kNoAllocBlock) k_noalloc_prepare(CountGrid g, 
     r.flags = kRayValid | (sample ? kRaySample : 0) | (M << kRayAxisShift);
     ray_constants(qo, qe, F, &r);
     r.inv = reciprocal64((unsigned long long)(M == 0 ? r.A[0] : (M == 1 ? r.A[1] : r.A[2])));
+    pieces = (M == 0 ? r.n[0] : (M == 1 ? r.n[1] : r.n[2])) / kNoAllocSlots + 1;
   }
-  rays[i] = r;
+  if (i < a.n) rays[i] = r;
+  pieces = __reduce_max_sync(0xffffffffu, pieces);
+  if ((threadIdx.x & 31) == 0) warp_pieces[i >> 5] = pieces;
 }
 
 static __device__ __noinline__ int na_exact_pick(const RayRec* rp, int F, int32_t c0, int32_t c1, int32_t c2) {
@@ -195,14 +204,24 @@ __device__ __forceinline__ void na_walk_piece(const CountGrid& g, const RayRec* 
     }
   }
 }
-__global__ void __launch_bounds__(kNoAllocBlock) k_noalloc_walk(CountGrid g, const RayRec* rays, int n, int pieces,
-                                                                uint32_t* hits, uint32_t* misses) {
+// A row of blocks (blockIdx.y) per piece that the range allows, where two
+// device-fulls of blocks reach that far; else (kTurns) the rows take the pieces in
+// turn, each warp up to its longest ray's last piece, so that a generous
+// max_range costs nothing beside short rays: 30,000 rays of 3 m with a range of
+// 1 km took 243 us with a thread for every piece, and take 50 us, as with a range
+// of 9 m.  (In turn with rows for every piece: 1 us of 56 slower.)
+template <bool kTurns>
+__global__ void __launch_bounds__(kNoAllocBlock) k_noalloc_walk(CountGrid g, const RayRec* rays, const int32_t* warp_pieces,
+                                                                int n, int pieces, uint32_t* hits, uint32_t* misses) {
+  if (kTurns) pieces = warp_pieces[(blockIdx.x * kNoAllocBlock + threadIdx.x) >> 5];
   for (int p = blockIdx.y; p < pieces; p += gridDim.y) na_walk_piece(g, rays, n, p * kNoAllocSlots, hits, misses);
 }
 
-// Device address of the static array, looked up once per device.
+// Device address of the static array and the blocks of the walk a device holds
+// at a time, looked up once per device.
 std::mutex g_noalloc_mutex;
 void* g_noalloc_ptr[64] = {nullptr};
+int g_noalloc_resident[64] = {0};
 
 }  // namespace
 }  // namespace ohm
@@ -244,11 +263,12 @@ ohm_status ohm_count_rays_noalloc(const ohm_count_grid* grid, const float* origi
   const double scale = std::ldexp(1.0, grid->frac_bits) / grid->voxel_size;
   if (grid->max_range * scale >= std::ldexp(1.0, 30))
     return na_fail(OHM_ERR_INVALID, "count_rays_noalloc: max_range * 2^frac_bits / voxel_size must be < 2^30");
-  // segments per ray <= (max_range / voxel_size + 2) / S + 1; the table must hold n of them
+  // the call's size limit, in segments of S dominant-axis steps: a ray has at
+  // most (max_range / voxel_size + 2) / S + 1 of them
   const long long per_ray = (long long)std::ceil(grid->max_range / grid->voxel_size + 2.0) / S + 1;
   if (per_ray * n > kNoAllocMaxSegments)
-    return na_fail(OHM_ERR_INVALID, "count_rays_noalloc: n * segments per ray exceeds the static segment table (" +
-                                        std::to_string(kNoAllocMaxSegments) + "); raise segment_steps or lower n");
+    return na_fail(OHM_ERR_INVALID, "count_rays_noalloc: n * segments per ray (max_range in segment_steps) exceeds " +
+                                        std::to_string(kNoAllocMaxSegments) + "; raise segment_steps or lower n");
   if (n == 0) return OHM_OK;
   if (!origins || !endpoints || (n_origins != 1 && n_origins != n))
     return na_fail(OHM_ERR_INVALID, "count_rays_noalloc: bad origins / endpoints");
@@ -262,10 +282,15 @@ ohm_status ohm_count_rays_noalloc(const ohm_count_grid* grid, const float* origi
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64)
     return na_fail(OHM_ERR_CUDA, "count_rays_noalloc: no current device");
   void* scratch = nullptr;
+  int resident = 0;
   {
     std::lock_guard<std::mutex> lock(g_noalloc_mutex);
     if (!g_noalloc_ptr[dev]) {
       // First call on this device: resolve the static array's device address.
+      int sms = 0, per_sm = 0;
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_noalloc_walk<true>, kNoAllocBlock, 0);
+      g_noalloc_resident[dev] = (sms > 0 ? sms : 1) * (per_sm > 0 ? per_sm : 1);
       cudaError_t e = cudaGetSymbolAddress(&g_noalloc_ptr[dev], g_noalloc_scratch);
       if (e != cudaSuccess) {
         g_noalloc_ptr[dev] = nullptr;
@@ -273,6 +298,7 @@ ohm_status ohm_count_rays_noalloc(const ohm_count_grid* grid, const float* origi
       }
     }
     scratch = g_noalloc_ptr[dev];
+    resident = g_noalloc_resident[dev];
   }
   CountGrid g;
   for (int k = 0; k < 3; ++k) {
@@ -292,13 +318,15 @@ ohm_status ohm_count_rays_noalloc(const ohm_count_grid* grid, const float* origi
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const unsigned blocks = (unsigned)((n + kNoAllocBlock - 1) / kNoAllocBlock);
   // a ray takes at most max_range / voxel_size + 2 steps of its dominant axis
-  // (one slot more), at most 2^22 + 3 by the check above
+  // (one slot more)
   const long long slots = (long long)std::ceil(grid->max_range / grid->voxel_size + 2.0) + 1;
-  const long long pieces = (slots + kNoAllocSlots - 1) / kNoAllocSlots;
+  const long long pieces = (slots + kNoAllocSlots - 1) / kNoAllocSlots, rows = 2LL * resident / blocks + 1;
   RayRec* rays = static_cast<RayRec*>(scratch);
-  k_noalloc_prepare<<<blocks, kNoAllocBlock, 0, s>>>(g, a, rays);
-  k_noalloc_walk<<<dim3(blocks, (unsigned)(pieces < 65535 ? pieces : 65535)), kNoAllocBlock, 0, s>>>(
-      g, rays, (int)n, (int)pieces, hits, misses);
+  int32_t* warp_pieces = reinterpret_cast<int32_t*>(static_cast<unsigned char*>(scratch) + kNoAllocRayBytes);
+  k_noalloc_prepare<<<blocks, kNoAllocBlock, 0, s>>>(g, a, rays, warp_pieces);
+  const auto walk = pieces <= rows ? k_noalloc_walk<false> : k_noalloc_walk<true>;
+  walk<<<dim3(blocks, (unsigned)std::min(pieces, rows)), kNoAllocBlock, 0, s>>>(g, rays, warp_pieces, (int)n, (int)pieces,
+                                                                                hits, misses);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return na_fail(OHM_ERR_CUDA, std::string("count_rays_noalloc: launch: ") + cudaGetErrorString(e));
   return OHM_OK;
