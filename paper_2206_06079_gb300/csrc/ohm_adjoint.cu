@@ -384,7 +384,9 @@ __global__ void __launch_bounds__(kBlock) k_ndt_backward(DeviceMap m, CallArgs a
       const int32_t slot = region_slot_of(m, v[0], v[1], v[2]);
       const int32_t ns = slot < 0 ? -1 : m.ndt_slot[slot];
       if (ns < 0) {
-        atomicOr(m.status, kStatusMissing);
+        // no end kernel follows: the host's word is written here
+        const int32_t status = atomicOr(m.status, kStatusMissing);
+        if (!(status & kStatusMissing)) *(volatile int32_t*)m.host_status = status | kStatusMissing;
       } else {
         const uint32_t mo = local_morton(v[0], v[1], v[2]);
         const uint32_t row = m.ndt_grad_row[voxel_offset(ns, mo)];  // 0: no query fell into the voxel
@@ -760,7 +762,6 @@ ohm_status ohm_ndt_backward(ohm_map* map, const double* pose, const float* origi
     k_ndt_grad_scatter<<<qb, kBlock, 0, s>>>(map->d, query_points, grad_mean, grad_cov, n_query, rows.p, rows.by_voxel, 0);
     map->launches += 1;
   }
-  map->status_copied = false;  // k_ndt_backward can latch a failure
   if (e == cudaSuccess && n > 0) {
     CallArgs a;
     e = stage_posed(map, P, origins, n_origins, endpoints, flags, n, s, &a);

@@ -294,13 +294,13 @@ ohm_status ohm_map_create(const ohm_map_params* params, ohm_map** out) {
   }
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&m->copy_stream, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m->work_done, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&m->h_status), 2 * sizeof(int32_t));
+  if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&m->h_status), sizeof(int32_t));
   if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&m->h_calls), sizeof(ohm::CallCounters));
   if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&m->h_count), 2 * sizeof(int32_t));
   if (e == cudaSuccess) {
     // ready for the first call (number 1; nothing is born in call 0)
-    m->h_status[0] = m->h_status[1] = 0;
-    d.host_status = m->h_status + 1;  // pinned memory is mapped at the same address
+    *m->h_status = 0;
+    d.host_status = m->h_status;  // pinned memory is mapped at the same address
     std::memset(m->h_calls, 0, sizeof(ohm::CallCounters));
     m->h_calls->seq = 1;
     e = cudaMemcpy(d.calls, m->h_calls, sizeof(ohm::CallCounters), cudaMemcpyHostToDevice);
@@ -374,17 +374,14 @@ ohm_status ohm_map_sync(ohm_map* map, void* stream) {
   if (!map) return fail(OHM_ERR_INVALID, "sync: map is NULL");
   DeviceGuard guard(map->device);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // The last kernel of every integrate call writes the status to pinned host
-  // memory; only after other work that can latch one is the word copied (a
-  // copy on the stream takes about 4 us of a call that waits).
-  const bool copy = !map->status_copied;
-  cudaError_t e = cudaSuccess;
-  if (copy) e = cudaMemcpyAsync(map->h_status, map->d.status, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  // The device writes a failed call's status to pinned host memory too: the
+  // last kernel of every integrate call, and the NDT adjoint (a copy on the
+  // stream takes about 4 us of a call that waits).
+  cudaError_t e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(e, "sync");
-  const int bits = *(volatile int32_t*)(map->h_status + (copy ? 0 : 1));
+  const int bits = *(volatile int32_t*)map->h_status;
   if (bits != 0) {
-    *(volatile int32_t*)(map->h_status + 1) = 0;
+    *(volatile int32_t*)map->h_status = 0;
     e = cudaMemsetAsync(map->d.status, 0, sizeof(int32_t), s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(e, "sync: clear status");

@@ -36,8 +36,7 @@ struct ohm_map {
   cudaEvent_t hin_free[2];    // kernels of the slot's last call done
   int hin_next;
   // pinned host mirrors for status / counters
-  int32_t* h_status;        // [0] copies of the device word, [1] DeviceMap::host_status
-  bool status_copied;       // h_status[1] holds (once the stream has passed) what the device word holds
+  int32_t* h_status;        // DeviceMap::host_status
   ohm::CallCounters* h_calls;
   int32_t* h_count;
   // rows of the backward calls' weights (take_rows), all zero between calls: the

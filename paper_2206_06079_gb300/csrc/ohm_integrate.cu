@@ -377,7 +377,6 @@ cudaError_t launch_integrate(ohm_map* map, const CallArgs& args, cudaStream_t st
   const int ray_grid = (int)(per_ray_blocks < grid ? per_ray_blocks : grid);
   const unsigned prb = (unsigned)per_ray_blocks;
   map->last_rays = n;
-  map->status_copied = true;
   if (occ_like) {
     if (n <= (long long)map->num_sms * OHM_PREPARE_MIN_BLOCKS * kBlock) {
       const unsigned wave_blocks = (unsigned)((n + kPrepareWaveBlock - 1) / kPrepareWaveBlock);
