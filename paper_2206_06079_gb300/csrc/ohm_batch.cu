@@ -243,14 +243,14 @@ __global__ void __launch_bounds__(kBlock) k_batch_tsdf_apply(const BatchDesc* de
 
 // One group of blocks per map rolls back that map if its call failed, and
 // makes its counters ready for the next call.
-__global__ void k_batch_end(const BatchDesc* desc) {
+__global__ void k_batch_end(const BatchDesc* desc, const BatchStep* step) {
   chain_enter();
   const int per_map = gridDim.x / kMaxBatchMaps;
   const int mi = blockIdx.x / per_map;
   if (mi >= desc->n_maps) return;
   const DeviceMap& m = desc->maps[mi];
   const long long b = blockIdx.x % per_map;
-  if (b == 0 && threadIdx.x == 0) finish_call(m);
+  if (b == 0 && threadIdx.x == 0) finish_call(m, step->n[mi]);
   if (!latched(m)) return;
   rollback_call(m, b * blockDim.x + threadIdx.x, (long long)per_map * blockDim.x);
 }
@@ -343,7 +343,7 @@ cudaError_t enqueue_step(ohm_batch* b, cudaStream_t s, int* count) {
     launch_chained(k_batch_tsdf_apply, ray_grid, s, b->d_desc, b->d_step);
     n += 2;
   }
-  launch_chained(k_batch_end, kMaxBatchMaps * 8, s, b->d_desc);
+  launch_chained(k_batch_end, kMaxBatchMaps * 8, s, b->d_desc, b->d_step);
   ++n;
   *count = n;
   return cudaGetLastError();
@@ -491,10 +491,7 @@ ohm_status ohm_batch_integrate(ohm_batch* b, const float* const* origins, const 
     }
   }
   if (e != cudaSuccess) return bfail(OHM_ERR_CUDA, std::string("batch_integrate: ") + cudaGetErrorString(e));
-  for (int i = 0; i < b->n_maps; ++i) {
-    b->maps[i]->last_rays = n[i];
-    ohm::note_work(b->maps[i], s);
-  }
+  for (int i = 0; i < b->n_maps; ++i) ohm::note_work(b->maps[i], s);
   return OHM_OK;
 }
 

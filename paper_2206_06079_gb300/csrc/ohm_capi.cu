@@ -602,7 +602,7 @@ ohm_status ohm_map_stats(ohm_map* map, ohm_call_stats* out, void* stream) {
     e = cudaMemcpyAsync(map->h_count + 1, map->d.ndt_count, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(e, "stats");
-  out->rays = (int64_t)map->last_rays;
+  out->rays = (int64_t)map->h_calls->last.rays;
   out->segments = (int64_t)map->h_calls->last.segments;
   out->visits = (int64_t)map->h_calls->last.visits;
   out->touched = (int64_t)map->h_calls->last.touched;

@@ -123,7 +123,7 @@ struct CallCounters {
   int32_t ndt_free_used_start;
   unsigned long long total_visits;  // every call since the map was made
   struct {
-    unsigned long long segments, visits, touched, atomics, restores;
+    unsigned long long rays, segments, visits, touched, atomics, restores;
   } last;                           // of the last finished call
 };
 

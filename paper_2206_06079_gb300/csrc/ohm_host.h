@@ -44,7 +44,6 @@ struct ohm_map {
   std::vector<double*> rows;
   long long rows_cap;       // doubles in the last of them
   long long launches;       // kernels launched by this map
-  long long last_rays;      // rays of the last integrate call
   // per-stage event timing
   uint32_t profile_mask;
   int32_t profile_every;    // record only every profile_every-th call (0 or 1: every call)

@@ -125,9 +125,9 @@ __global__ void __launch_bounds__(kBlock) k_tsdf_apply(DeviceMap m) {
   OHM_GRID_STRIDE(t, nt) tsdf_apply_one(m, t);
 }
 
-__global__ void k_end(DeviceMap m) {
+__global__ void k_end(DeviceMap m, long long n) {
   chain_enter();
-  if (blockIdx.x == 0 && threadIdx.x == 0) finish_call(m);
+  if (blockIdx.x == 0 && threadIdx.x == 0) finish_call(m, n);
   if (!latched(m)) return;
   rollback_call(m, (long long)blockIdx.x * blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
 }
@@ -376,7 +376,6 @@ cudaError_t launch_integrate(ohm_map* map, const CallArgs& args, cudaStream_t st
   const long long per_ray_blocks = blocks_for(n) > 0 ? blocks_for(n) : 1;
   const int ray_grid = (int)(per_ray_blocks < grid ? per_ray_blocks : grid);
   const unsigned prb = (unsigned)per_ray_blocks;
-  map->last_rays = n;
   if (occ_like) {
     if (n <= (long long)map->num_sms * OHM_PREPARE_MIN_BLOCKS * kBlock) {
       const unsigned wave_blocks = (unsigned)((n + kPrepareWaveBlock - 1) / kPrepareWaveBlock);
@@ -414,7 +413,7 @@ cudaError_t launch_integrate(ohm_map* map, const CallArgs& args, cudaStream_t st
     OHM_LAUNCH(OHM_STAGE_TSDF_APPLY, launch_chained(k_tsdf_apply, grid, stream, m));
   }
   // one block per SM: the body only runs (a grid-stride rollback) after a failure
-  OHM_LAUNCH(OHM_STAGE_END, launch_chained(k_end, (unsigned)map->num_sms, stream, m));
+  OHM_LAUNCH(OHM_STAGE_END, launch_chained(k_end, (unsigned)map->num_sms, stream, m, n));
   return cudaGetLastError();
 }
 

@@ -310,7 +310,7 @@ __device__ __forceinline__ void snapshot_pool(const DeviceMap& m) {
 // goes out before the first store, and the host's word, which ohm_map_sync
 // reads (and zeroes) without a copy of its own, is written after a failure
 // only.
-__device__ __forceinline__ void finish_call(const DeviceMap& m) {
+__device__ __forceinline__ void finish_call(const DeviceMap& m, long long rays) {
   CallCounters* c = m.calls;
   const auto segments = c->segments;
   const auto visits = c->visits;
@@ -324,6 +324,7 @@ __device__ __forceinline__ void finish_call(const DeviceMap& m) {
   const auto free_used = m.free_info[1];
   const auto ndt_free_used = m.free_info[3];
   const int32_t status = *(volatile int32_t*)m.status;
+  c->last.rays = (unsigned long long)rays;
   c->last.segments = segments;
   c->last.visits = visits;
   c->last.touched = touched;

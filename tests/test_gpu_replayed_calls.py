@@ -48,3 +48,23 @@ def test_sync_reports_a_failure_of_a_replayed_backward():
         m.sync()  # reported once
         m.integrate(o, e)
 
+
+
+def test_stats_of_a_replayed_call():
+    with _map() as m:
+        o, e = _rays(500, [1.6, 1.6, 1.6])
+        m.integrate(o, e)
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            m.integrate(o, e, sync=False)
+        few = e[:100].contiguous()
+        m.integrate(o, few)
+        assert m.stats()["rays"] == 100
+        g.replay()
+        s = m.stats()
+        assert s["rays"] == 500 and s["visits"] > 500
+        batch = ohm.Batch([m])
+        batch.integrate([(o, few, None)], graph=False)
+        batch.sync()
+        assert m.stats()["rays"] == 100
+        batch.close()
