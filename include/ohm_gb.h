@@ -306,8 +306,8 @@ typedef enum {
   OHM_STAGE_HITS = 5,         /* sample updates and NDT moments (phase two) */
   OHM_STAGE_TSDF_WALK = 6,    /* TSDF band walk */
   OHM_STAGE_TSDF_APPLY = 7,   /* TSDF weighted average */
-  OHM_STAGE_END = 8,          /* rollback of a failed call, rollback snapshot and counters of the
-                                 next call, status copy */
+  OHM_STAGE_END = 8,          /* rollback of a failed call and its status in host memory, rollback
+                                 snapshot and counters of the next call */
   OHM_STAGE_MEAN_APPLY = 9,   /* voxel-mean per-call update */
   OHM_STAGE_COUNT = 10
 } ohm_stage;

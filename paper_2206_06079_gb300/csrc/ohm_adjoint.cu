@@ -158,19 +158,34 @@ __device__ __forceinline__ long long claim_row(uint32_t* plane, long long off, l
 }
 
 // The upstream weight G(v) of a voxel, the sum of g_q over the queries it
-// holds: a row of one double, added to for each query point, or (clear) zeroed
-// and forgotten.
+// holds, in three passes over the queries: add them up in rows of one double
+// (row[q]: the row of query q; by_voxel: the voxel's own), put each voxel's sum
+// into its word as a float, and, after the backward pass, zero everything.
+// The backward pass reads a float per band voxel: with the row in the word and the
+// sum behind it, the call took 102 us for a 640 x 480 frame at 5 cm and 130 at
+// 2 cm; with the second pass 101 and 122, with the four kernels chained 99 and 118
+// (float atomics straight into the words: 94 and 115).
+enum GradPass { kGradAdd, kGradSettle, kGradClear };
+template <GradPass kPass>
 __global__ void __launch_bounds__(kBlock) k_grad_scatter(DeviceMap m, const float* pts, const float* g, long long n,
-                                                         double* rows, int by_voxel, int clear) {
+                                                         double* rows, uint32_t* row, int by_voxel) {
+  chain_enter();
   for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x) {
     const long long off = point_offset(m, pts + 3 * q);
     if (off < 0) continue;
-    if (clear) {
-      const uint32_t row = m.grad_row[off];  // 0: another query of the voxel was here
-      if (row) rows[row - 1u] = 0.0;
-      m.grad_row[off] = 0u;
+    long long r = off;
+    if (kPass == kGradAdd) {
+      if (!by_voxel) row[q] = (uint32_t)(r = claim_row(m.grad, off, q));
+      atomicAdd(rows + r, (double)g[q]);
+      continue;
+    }
+    if (!by_voxel) r = row[q];
+    if (kPass == kGradSettle) {
+      m.grad[off] = __float_as_uint((float)rows[r]);
     } else {
-      atomicAdd(rows + claim_row(m.grad_row, off, by_voxel ? off : q), (double)g[q]);
+      if (!by_voxel) row[q] = 0u;
+      rows[r] = 0.0;
+      m.grad[off] = 0u;
     }
   }
 }
@@ -182,10 +197,12 @@ __device__ __forceinline__ double warp_sum(double v) {
 }
 
 // Compiled for 2 blocks per SM (128 registers; 184 unbounded, which fits one;
-// 3 and 4 blocks: no difference).  640 x 480 frame with 20,000 queries: 121 us with
-// the double back-projection and the 64-bit walker, row by row; 100 us now.
-__global__ void __launch_bounds__(kBlock, 2) k_tsdf_backward(DeviceMap m, DepthFrame f, const double* rows,
-                                                          float* grad_depth, double* grad_twist) {
+// 3 and 4 blocks: no difference).  Bound by instruction issue.  The whole call for
+// a 640 x 480 frame with 20,000 queries: 121 us with the double back-projection and
+// the 64-bit walker, row by row; 99 us now.
+__global__ void __launch_bounds__(kBlock, 2) k_tsdf_backward(DeviceMap m, DepthFrame f, float* grad_depth,
+                                                          double* grad_twist) {
+  chain_enter();
   __shared__ double red[kBlock / 32][6];
   __shared__ uint32_t tabs[8 * kBlock];
   uint32_t* const tab = tabs + threadIdx.x;
@@ -224,13 +241,11 @@ __global__ void __launch_bounds__(kBlock, 2) k_tsdf_backward(DeviceMap m, DepthF
 #pragma unroll
         for (int k = 0; k < 3; ++k) rel[k] = t.e[k] - ((ps.v[k] - t.r.v0[k]) << F);
         for (left = ps.visits; left > 0;) {
-          uint32_t at[kFastBatch], off[kFastBatch], row[kFastBatch], valid;
+          uint32_t at[kFastBatch], off[kFastBatch], valid;
           float G[kFastBatch];
           piece_fill<true>(m, &t.r, K, tab, w, mo, left, at, off, valid);
 #pragma unroll
-          for (int j = 0; j < kFastBatch; ++j) row[j] = ((valid >> j) & 1u) ? m.grad_row[off[j]] : 0u;
-#pragma unroll
-          for (int j = 0; j < kFastBatch; ++j) G[j] = row[j] ? (float)rows[row[j] - 1u] : 0.f;
+          for (int j = 0; j < kFastBatch; ++j) G[j] = ((valid >> j) & 1u) ? __uint_as_float(m.grad[off[j]]) : 0.f;
 #pragma unroll
           for (int j = 0; j < kFastBatch; ++j) {
             if (G[j] != 0.f) {
@@ -508,19 +523,21 @@ cudaError_t frame_tables(ohm_map* map, DepthFrame* f, cudaStream_t s) {
 }
 
 // Zeroed rows of `width` doubles for a backward call's queries (claim_row), one
-// per query or, where there are fewer, per voxel of the layer.  The buffer stays
-// with the map and the clearing pass zeroes what the call used, so that a call
-// costs no allocation and no fill (a pool allocation and a fill for each call
-// took 12 to 30 us of 510).  It grows by doubling; a captured call that finds it
-// too small takes memory that its graph then holds (`own`).
+// per query (and `extra` doubles behind them) or, where there are fewer, per
+// voxel of the layer.  The buffer stays with the map and the clearing pass zeroes
+// what the call used, so that a call costs no allocation and no fill (a pool
+// allocation and a fill for each call took 12 to 30 us of 510).  It grows by
+// doubling; a captured call that finds it too small takes memory that its graph
+// then holds (`own`).
 struct Rows {
   double* p = nullptr;
   int by_voxel = 0;
   bool own = false;
 };
-cudaError_t take_rows(ohm_map* map, long long n_query, long long voxels, int width, cudaStream_t s, Rows* r) {
+cudaError_t take_rows(ohm_map* map, long long n_query, long long voxels, int width, long long extra, cudaStream_t s,
+                      Rows* r) {
   r->by_voxel = n_query > voxels ? 1 : 0;
-  const long long need = width * (r->by_voxel ? voxels : n_query);
+  const long long need = r->by_voxel ? width * voxels : width * n_query + extra;
   if (need <= map->rows_cap) {
     r->p = map->rows.back();
     return cudaSuccess;
@@ -631,10 +648,10 @@ ohm_status ohm_tsdf_backward(ohm_map* map, const float* depth, int32_t width, in
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   cudaError_t e = cudaSuccess;
   const long long voxels = (long long)map->p.max_regions * kRegionVoxels;
-  if (!map->d.grad_row) {
-    // rows of upstream weights per voxel, allocated on the first backward call
-    e = cudaMalloc(reinterpret_cast<void**>(&map->d.grad_row), sizeof(uint32_t) * (size_t)voxels);
-    if (e == cudaSuccess) e = cudaMemsetAsync(map->d.grad_row, 0, sizeof(uint32_t) * (size_t)voxels, s);
+  if (!map->d.grad) {
+    // upstream weights per voxel, allocated on the first backward call
+    e = cudaMalloc(reinterpret_cast<void**>(&map->d.grad), sizeof(uint32_t) * (size_t)voxels);
+    if (e == cudaSuccess) e = cudaMemsetAsync(map->d.grad, 0, sizeof(uint32_t) * (size_t)voxels, s);
   }
   const long long n = (long long)width * height;
   const int qb = (int)(n_query > 0 ? ((n_query + kBlock - 1) / kBlock < 4096 ? (n_query + kBlock - 1) / kBlock : 4096) : 0);
@@ -642,18 +659,20 @@ ohm_status ohm_tsdf_backward(ohm_map* map, const float* depth, int32_t width, in
   if (e == cudaSuccess) e = frame_tables(map, &f, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(grad_twist, 0, 6 * sizeof(double), s);
   Rows rows;
-  if (e == cudaSuccess && qb) e = take_rows(map, n_query, voxels, 1, s, &rows);
+  if (e == cudaSuccess && qb) e = take_rows(map, n_query, voxels, 1, (n_query + 1) / 2, s, &rows);
+  uint32_t* const row = rows.p && !rows.by_voxel ? reinterpret_cast<uint32_t*>(rows.p + n_query) : nullptr;
   if (e == cudaSuccess && qb) {
-    k_grad_scatter<<<qb, kBlock, 0, s>>>(map->d, query_points, grad_query, n_query, rows.p, rows.by_voxel, 0);
-    map->launches += 1;
+    launch_chained(k_grad_scatter<kGradAdd>, qb, s, map->d, query_points, grad_query, n_query, rows.p, row, rows.by_voxel);
+    launch_chained(k_grad_scatter<kGradSettle>, qb, s, map->d, query_points, grad_query, n_query, rows.p, row, rows.by_voxel);
+    map->launches += 2;
   }
   if (e == cudaSuccess) {
-    k_tsdf_backward<<<pb, kBlock, 0, s>>>(map->d, f, rows.p, grad_depth, grad_twist);
+    launch_chained(k_tsdf_backward, pb, s, map->d, f, grad_depth, grad_twist);
     map->launches += 1;
   }
   if (rows.p) {
     // whatever else failed: no row may outlive its call in the plane
-    k_grad_scatter<<<qb, kBlock, 0, s>>>(map->d, query_points, grad_query, n_query, rows.p, rows.by_voxel, 1);
+    launch_chained(k_grad_scatter<kGradClear>, qb, s, map->d, query_points, grad_query, n_query, rows.p, row, rows.by_voxel);
     map->launches += 1;
     const cudaError_t ef = give_rows(rows, s);
     if (e == cudaSuccess) e = ef;
@@ -757,7 +776,7 @@ ohm_status ohm_ndt_backward(ohm_map* map, const double* pose, const float* origi
   if (e == cudaSuccess) e = cudaMemsetAsync(grad_twist, 0, 6 * sizeof(double), s);
   const int qb = (int)(n_query > 0 ? ((n_query + kBlock - 1) / kBlock < 4096 ? (n_query + kBlock - 1) / kBlock : 4096) : 0);
   Rows rows;
-  if (e == cudaSuccess && qb) e = take_rows(map, n_query, voxels, 9, s, &rows);
+  if (e == cudaSuccess && qb) e = take_rows(map, n_query, voxels, 9, 0, s, &rows);
   if (e == cudaSuccess && qb) {
     k_ndt_grad_scatter<<<qb, kBlock, 0, s>>>(map->d, query_points, grad_mean, grad_cov, n_query, rows.p, rows.by_voxel, 0);
     map->launches += 1;

@@ -75,7 +75,7 @@ void free_map(ohm_map* m) {
   if (!m) return;
   ohm::DeviceMap& d = m->d;
   void* ptrs[] = {d.htab, d.region_count, d.region_coords, d.occ, d.sat, d.counts, d.decay, d.vmean, d.vmean_acc, d.mean_list, d.ndt_slot, d.ndt_count, d.ndt_pending,
-                  d.ndt, d.tsdf, d.tsdf_cnt, d.tsdf_sum, d.grad_row, d.ndt_grad_row, d.status, d.calls, d.rays, d.decay_rays, d.trays, d.segs, d.touched,
+                  d.ndt, d.tsdf, d.tsdf_cnt, d.tsdf_sum, d.grad, d.ndt_grad_row, d.status, d.calls, d.rays, d.decay_rays, d.trays, d.segs, d.touched,
                   d.stamp, d.born, d.ndt_born, d.free_slots, d.ndt_free, d.free_info, d.restore_keys,
                   m->stage_origins, m->stage_endpoints, m->stage_flags, m->hin_origins[0], m->hin_origins[1],
                   m->hin_endpoints[0], m->hin_endpoints[1], m->hin_flags[0], m->hin_flags[1], m->pxy};

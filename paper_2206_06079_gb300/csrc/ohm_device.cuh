@@ -94,7 +94,6 @@ struct __align__(16) TsdfRec {
   float u[3];       // unit direction sensor -> sample
 };
 
-// Per-call counters in device memory.
 // A float-float value hi + lo with |lo| <= ulp(hi) / 2 (the arithmetic is
 // with the TSDF band below).
 struct FF {
@@ -106,8 +105,8 @@ struct BandConsts {
   FF tau, rmin, rmax;  // fixed-point units
 };
 
-// Between calls they stand ready for the next one: k_end moves the finished
-// call's values to `last`, zeroes them and takes the pool snapshot.
+// Per-call counters in device memory.  Between calls they stand ready for the
+// next one: k_end moves the finished call's values to `last`, zeroes them and takes the pool snapshot.
 struct CallCounters {
   unsigned long long segments;
   unsigned long long visits;
@@ -153,8 +152,9 @@ struct DeviceMap {
   float2* tsdf;                  // [max_regions][32768] (D, W)
   uint32_t* tsdf_cnt;            // [max_regions][32768] per-call scratch, zero between calls
   long long* tsdf_sum;           // [max_regions][32768] per-call scratch, 2^-32 m units
-  uint32_t* grad_row;            // [max_regions][32768] row of a voxel's TSDF adjoint weight plus one, zero between calls;
-                                 // allocated by the first backward call
+  uint32_t* grad;                // [max_regions][32768] row of a voxel's TSDF adjoint weight plus one while the weights
+                                 // are summed, then the weight (float bits); zero between calls; allocated by the
+                                 // first backward call
   uint32_t* ndt_grad_row;        // [max_ndt][32768] row of a voxel's NDT adjoint weights plus one, zero between calls;
                                  // allocated by the first NDT backward call
   int32_t* status;
@@ -350,7 +350,8 @@ __host__ __device__ __forceinline__ uint32_t region_morton(int32_t vx, int32_t v
   return morton((uint32_t)(vx & mask), (uint32_t)(vy & mask), (uint32_t)(vz & mask));
 }
 
-// Step one axis of a Morton index by +-1, wrapping inside the 5 bits of that axis.
+// Step one axis of a Morton index by +-1, wrapping inside the 5 bits of that axis
+// (host tests only: the local walk steps six bits per axis).
 __host__ __device__ __forceinline__ uint32_t morton_step(uint32_t m, uint32_t mask, int sign) {
   uint32_t moved = sign > 0 ? ((m | ~mask) + 1u) : ((m & mask) - 1u);
   return (moved & mask) | (m & ~mask);
@@ -398,8 +399,8 @@ __host__ __device__ __forceinline__ long long sel3(int k, long long a, long long
   return k == 0 ? a : (k == 1 ? b : c);
 }
 
-// Returns the index of the dominant axis (the lowest of equal ones) and the
-// number of steps it takes.
+// Returns the index of the axis with the most voxel steps (the lowest of equal
+// ones) and their number (host tests only: the kernels' rays go by longest_axis).
 __host__ __device__ __forceinline__ int dominant_axis(const long long a[3], const long long b[3], int F, int32_t* nmaj) {
   long long d0 = (b[0] >> F) - (a[0] >> F), d1 = (b[1] >> F) - (a[1] >> F), d2 = (b[2] >> F) - (a[2] >> F);
   d0 = d0 < 0 ? -d0 : d0;
@@ -548,7 +549,8 @@ OHM_UNROLL
   }
 }
 
-// walker_init from the per-ray constants (same state, cheaper set-up).
+// walker_init from the per-ray constants (same state, cheaper set-up; host tests
+// only).
 __host__ __device__ inline void walker_init_rec(Walker& w, const RayRec& r, int F, int M, long long K) {
   const long long U = 1LL << F;
   const long long d0M = M == 0 ? r.d0[0] : (M == 1 ? r.d0[1] : r.d0[2]);
@@ -617,8 +619,10 @@ __host__ __device__ __forceinline__ uint32_t morton_mask(int axis) {
 }
 
 // ---------------------------------------------------------------------------
-// Filtered exact walk: the integrate kernels' voxel walk.  It visits exactly
-// the voxels of Walker, in the same order, with cheaper steps.
+// Filtered exact walk: what the integrate kernels walked before the local walk
+// (LWalker, below).  No kernel runs it any more; the host walker test holds it,
+// SegStart and the Morton stepping beside it against the oracle.  It visits
+// exactly the voxels of Walker, in the same order, with cheaper steps.
 //
 // Along every axis k it keeps c_k, the boundary crossings taken so far, and
 // an FP32 estimate of the exact crossing parameter of the next boundary,
@@ -767,7 +771,7 @@ __host__ __device__ __forceinline__ bool morton_advance(uint32_t& mo, uint32_t m
 
 
 // Number of segments of a walk whose dominant axis takes nmaj steps, cut
-// every S dominant-axis steps (the allocation-free entry point's split).
+// every S dominant-axis steps (host tests only).
 __host__ __device__ __forceinline__ int32_t segment_count(int32_t nmaj, int32_t S) { return nmaj / S + 1; }
 
 // Ray segments of the integrate kernels (Sec. III-B "breaking long rays into
@@ -811,7 +815,8 @@ __host__ __device__ __forceinline__ void segment_bounds(int32_t nmaj, int32_t ns
 }
 constexpr int kRaySegShift = 16;  // RayRec flags bits 16..31: q, the ray's dominant-axis slots per segment
 
-// Where segment j of a ray starts and ends, for the filtered walk.
+// Where segment j of a ray starts and ends, for the filtered walk (host tests
+// only; the kernels' pieces start with piece_start).
 struct SegStart {
   long long c[3];    // crossings taken along each axis before the segment's first voxel
   int32_t v[3];      // the segment's first voxel
@@ -1314,7 +1319,7 @@ __host__ __device__ __forceinline__ FF ff_of_int(int32_t v) {
   return {hi, (float)(v - (int32_t)hi)};
 }
 
-// rint(s) of a float-float s with |s| < 2^27, as ff_rint (below) does for
+// rint(s) of a float-float s with |s| < 2^27, as ff_rint (above) does for
 // |x| < 2^25: the low part may itself be a few units.
 __host__ __device__ __forceinline__ bool ff_rint_wide(FF s, float e, int32_t* out) {
   const float n = rintf(s.hi);

@@ -29,7 +29,7 @@ namespace ohm {
 // lookups, so in a call that fits one wave the SM with the most rays ends it.
 // Blocks of 128 rays share such a call out more evenly than blocks of 256 (131,072
 // rays on 152 SMs: at most 7 x 128 a SM instead of 4 x 256): a tunnel scan
-// 51.0 -> 47.6 us, outdoors 35.5 -> 33.8.  A call of several waves is faster in
+// 51.0 -> 47.2 us, outdoors 35.5 -> 34.9.  A call of several waves is faster in
 // blocks of 256 (262,144 rays: 67.3 against 72.7 us).
 constexpr int kPrepareWaveBlock = 128;
 template <int kThreads>

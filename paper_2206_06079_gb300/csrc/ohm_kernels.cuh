@@ -672,7 +672,7 @@ __device__ __forceinline__ bool miss_add(float* occ, uint32_t off, uint32_t& wor
 }
 
 // Look at the warp's waiting voxels and give them their misses, until fewer
-// than `keep` + 1 wait; four per lane at a time.  Returns the log-odds atomics
+// than `keep` wait; four per lane at a time.  Returns the log-odds atomics
 // this lane issued.  Whole warps; out of line: a well observed map comes here
 // about once per six rounds of segments.
 static __device__ __noinline__ unsigned int drain_open(float* occ_any, uint32_t* sat_any, float miss, float l_min,
@@ -1262,9 +1262,9 @@ __device__ __forceinline__ void prepare_tsdf_ray(const DeviceMap& m, const CallA
 // reveal are appended to the touched list with one atomic per warp and batch.
 // Measured on 640 x 480 frames at 5 cm: 72 us with the 64-bit walker, rows of 32
 // pixels per warp and each group's leader adding up its lanes; with the local
-// walk and 8 x 4 pixel tiles 106 us in that form, 96 us reducing up to six
-// groups, 56 us with shared sums alone, 41 us compiled for 4 blocks per SM (the
-// launch's two full waves), 40 us in this form.
+// walk and 8 x 4 pixel tiles 106 us in that form, 80 / 96 / 209 us reducing up to 3 /
+// 6 / 12 groups, 56 us with shared sums alone, 41 us compiled for 4 blocks per SM
+// (the launch's two full waves), 40 us in this form.
 constexpr int kTsdfReduce = 8;
 __device__ __forceinline__ void tsdf_walk_ray(const DeviceMap& m, long long i, bool active, uint32_t* tab,
                                               uint32_t* acc) {
