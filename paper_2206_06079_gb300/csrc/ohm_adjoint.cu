@@ -534,12 +534,12 @@ struct Rows {
   int by_voxel = 0;
   bool own = false;
 };
-cudaError_t take_rows(ohm_map* map, long long n_query, long long voxels, int width, long long extra, cudaStream_t s,
+cudaError_t take_rows(RowBuffers& kept, long long n_query, long long voxels, int width, long long extra, cudaStream_t s,
                       Rows* r) {
   r->by_voxel = n_query > voxels ? 1 : 0;
   const long long need = r->by_voxel ? width * voxels : width * n_query + extra;
-  if (need <= map->rows_cap) {
-    r->p = map->rows.back();
+  if (need <= kept.cap) {
+    r->p = kept.all.back();
     return cudaSuccess;
   }
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
@@ -551,7 +551,7 @@ cudaError_t take_rows(ohm_map* map, long long n_query, long long voxels, int wid
     e = cudaMallocAsync(reinterpret_cast<void**>(&p), sizeof(double) * (size_t)need, s);
     r->own = e == cudaSuccess;
   } else {
-    cap = std::max(need, std::max(2 * map->rows_cap, 1LL << 16));
+    cap = std::max(need, std::max(2 * kept.cap, 1LL << 16));
     e = cudaMalloc(reinterpret_cast<void**>(&p), sizeof(double) * (size_t)cap);
   }
   if (e != cudaSuccess) return e;
@@ -561,8 +561,8 @@ cudaError_t take_rows(ohm_map* map, long long n_query, long long voxels, int wid
       cudaFree(p);
       return e;
     }
-    map->rows.push_back(p);
-    map->rows_cap = cap;
+    kept.all.push_back(p);
+    kept.cap = cap;
   }
   r->p = p;
   return e;
@@ -659,7 +659,7 @@ ohm_status ohm_tsdf_backward(ohm_map* map, const float* depth, int32_t width, in
   if (e == cudaSuccess) e = frame_tables(map, &f, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(grad_twist, 0, 6 * sizeof(double), s);
   Rows rows;
-  if (e == cudaSuccess && qb) e = take_rows(map, n_query, voxels, 1, (n_query + 1) / 2, s, &rows);
+  if (e == cudaSuccess && qb) e = take_rows(map->tsdf_rows, n_query, voxels, 1, (n_query + 1) / 2, s, &rows);
   uint32_t* const row = rows.p && !rows.by_voxel ? reinterpret_cast<uint32_t*>(rows.p + n_query) : nullptr;
   if (e == cudaSuccess && qb) {
     launch_chained(k_grad_scatter<kGradAdd>, qb, s, map->d, query_points, grad_query, n_query, rows.p, row, rows.by_voxel);
@@ -776,7 +776,7 @@ ohm_status ohm_ndt_backward(ohm_map* map, const double* pose, const float* origi
   if (e == cudaSuccess) e = cudaMemsetAsync(grad_twist, 0, 6 * sizeof(double), s);
   const int qb = (int)(n_query > 0 ? ((n_query + kBlock - 1) / kBlock < 4096 ? (n_query + kBlock - 1) / kBlock : 4096) : 0);
   Rows rows;
-  if (e == cudaSuccess && qb) e = take_rows(map, n_query, voxels, 9, 0, s, &rows);
+  if (e == cudaSuccess && qb) e = take_rows(map->ndt_rows, n_query, voxels, 9, 0, s, &rows);
   if (e == cudaSuccess && qb) {
     k_ndt_grad_scatter<<<qb, kBlock, 0, s>>>(map->d, query_points, grad_mean, grad_cov, n_query, rows.p, rows.by_voxel, 0);
     map->launches += 1;

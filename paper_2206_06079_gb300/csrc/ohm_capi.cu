@@ -89,7 +89,8 @@ void free_map(ohm_map* m) {
   ohm::destroy_host_store(m);
   for (void* p : ptrs)
     if (p) cudaFree(p);
-  for (double* r : m->rows) cudaFree(r);
+  for (const auto* rows : {&m->tsdf_rows, &m->ndt_rows})
+    for (double* r : rows->all) cudaFree(r);
   if (m->h_status) cudaFreeHost(m->h_status);
   if (m->h_calls) cudaFreeHost(m->h_calls);
   if (m->h_count) cudaFreeHost(m->h_count);

@@ -13,6 +13,11 @@
 
 namespace ohm {
 struct HostStore;
+// The last buffer is in use, smaller ones stay for graphs that captured them.
+struct RowBuffers {
+  std::vector<double*> all;
+  long long cap = 0;  // doubles in the last of them
+};
 }
 
 struct ohm_map {
@@ -39,10 +44,8 @@ struct ohm_map {
   int32_t* h_status;        // DeviceMap::host_status
   ohm::CallCounters* h_calls;
   int32_t* h_count;
-  // rows of the backward calls' weights (take_rows), all zero between calls: the
-  // last buffer is in use, smaller ones stay for graphs that captured them
-  std::vector<double*> rows;
-  long long rows_cap;       // doubles in the last of them
+  // rows of the backward calls' weights (take_rows), all zero between calls
+  ohm::RowBuffers tsdf_rows, ndt_rows;
   long long launches;       // kernels launched by this map
   // per-stage event timing
   uint32_t profile_mask;
