@@ -553,6 +553,11 @@ cudaError_t take_rows(RowBuffers& kept, long long n_query, long long voxels, int
   } else {
     cap = std::max(need, std::max(2 * kept.cap, 1LL << 16));
     e = cudaMalloc(reinterpret_cast<void**>(&p), sizeof(double) * (size_t)cap);
+    if (e == cudaErrorMemoryAllocation && cap > need) {  // no room to grow ahead
+      cudaGetLastError();
+      cap = need;
+      e = cudaMalloc(reinterpret_cast<void**>(&p), sizeof(double) * (size_t)cap);
+    }
   }
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(p, 0, sizeof(double) * (size_t)cap, s);
